@@ -281,7 +281,9 @@ int lbm_solver_set_kernel(lbm_solver *s, int32_t kernel, int32_t variant);
  * flag.  The state of that step is then incomplete: reload one (set_state,
  * set_f or init) before stepping on.  0 makes every such wait give up at
  * once, met or not (the failure path on demand; the drain before exit still
- * waits).  The other kernels have no waits.  Errors: LBM_EINVAL. */
+ * waits).  FP64 CELLWARP grids advance many steps per launch behind a grid
+ * barrier whose waits have a fixed 2 s limit and the same outcome; the other
+ * kernels have no waits.  Errors: LBM_EINVAL. */
 int lbm_solver_set_wait_limit(lbm_solver *s, uint64_t ns);
 /* Number of compiled variants of `kernel` (DIRECT or STAGED) for this
  * solver's precision.  Errors: LBM_EINVAL. */

@@ -1,8 +1,10 @@
 // C ABI of the library (include/lbm.h): handles, parameter checks, device
 // memory layout, and the host side of each call.  Every step of the method
 // runs in the CUDA kernels this file launches.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <new>
 #include <string>
@@ -265,6 +267,42 @@ void fill_consts(KConsts<C> &k, const LatticeHost &L, const lbm_params &p, int p
     }
 }
 
+void fill_cell_lanes(CellLanes &c, const LatticeHost &L, const lbm_params &p) {
+    std::memset(&c, 0, sizeof(c));
+    for (int l = 0; l <= (L.Q - 1) / 2; ++l) {
+        const int a = l ? 2 * l - 1 : 0;
+        const double c2 = L.r * L.r * (L.ex[a] * L.ex[a] + L.ey[a] * L.ey[a]);
+        c.ex[l] = (signed char)L.ex[a];
+        c.ey[l] = (signed char)L.ey[a];
+        c.cx[l] = L.r * L.ex[a];
+        c.cy[l] = L.r * L.ey[a];
+        c.x0[l] = c2 - 2;
+        c.x1[l] = -0.5 * (c2 - 4);
+        c.x2[l] = 0.25 * (c2 * c2 - 8 * c2 + 8);
+        c.t1[l] = 0.5 * (c2 - 4);
+        c.t2[l] = 0.5 * (c2 - 6);
+        c.we[l] = 0.5 * L.w[a];
+        c.wo[l] = L.w[a];
+    }
+    int nt[2] = {0, 0};
+    for (int a = 0; a < L.Q; ++a) {
+        c.mom[0][a] = 1.0;
+        c.mom[1][a] = L.r * L.ex[a];
+        c.mom[2][a] = L.r * L.ey[a];
+        c.mom[3][a] = 0.5 * L.r * L.r * (L.ex[a] * L.ex[a] + L.ey[a] * L.ey[a]);
+        const int wall = L.ey[a] < 0 ? 0 : 1;
+        for (int kk = 0; kk < std::abs(L.ey[a]); ++kk) {
+            c.tb[wall][nt[wall]] = (signed char)a;
+            c.tk[wall][nt[wall]] = (signed char)kk;
+            c.tx[wall][nt[wall]++] = (signed char)L.ex[a];
+        }
+    }
+    c.nterm = nt[0];                          // symmetric sets: the same for both walls, <= 26
+    c.tau_half = p.tau * L.r * p.Ny + 0.5;
+    c.diffuse[0] = p.accom[0] == 1.0;
+    c.diffuse[1] = p.accom[1] == 1.0;
+}
+
 template void fill_consts<float>(KConsts<float> &, const LatticeHost &, const lbm_params &, int);
 template void fill_consts<double>(KConsts<double> &, const LatticeHost &, const lbm_params &, int);
 
@@ -476,6 +514,7 @@ int lbm_solver_create(const lbm_lattice *lat, const lbm_params *p, void *stream,
     s.red_elems = lo.red_bytes / 8;
     s.derr = (int *)(s.red + 8 * 1024 + 48);
     s.sr = (unsigned *)(s.red + 8 * 1024 + 56);
+    s.bar = (unsigned *)(s.red + 8 * 1024 + 52);
     s.cur = 0;
     s.tm_key = -1;
     s.variant = 0;
@@ -484,7 +523,8 @@ int lbm_solver_create(const lbm_lattice *lat, const lbm_params *p, void *stream,
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&s.sm_count, cudaDevAttrMultiProcessorCount, dev);
         if (s.sm_count < 1) s.sm_count = 1;
-        cudaError_t e = cudaMemsetAsync(s.derr, 0, sizeof(int), s.stream);
+        // the error flag and the barrier words (derr .. sr)
+        cudaError_t e = cudaMemsetAsync(s.derr, 0, 8 * sizeof(double), s.stream);
         if (e != cudaSuccess) {
             if (s.owns_mem) cudaFreeAsync(s.dmem, s.stream);
             cudaFreeHost(s.pinned);
@@ -495,6 +535,7 @@ int lbm_solver_create(const lbm_lattice *lat, const lbm_params *p, void *stream,
     }
     fill_consts(s.kd, s.L, s.p, s.pitch);
     fill_consts(s.kf, s.L, s.p, s.pitch);
+    fill_cell_lanes(s.lanes, s.L, s.p);
     s.kd.f0 = s.kf.f0 = s.f[0];
     s.kd.sr = s.kf.sr = s.sr;
     s.last_res = -1;
@@ -598,6 +639,17 @@ int lbm_solver_step(lbm_solver *h, int64_t n) {
         return LBM_OK;
     };
     int rc;
+    while (n >= 2 && kern == LBM_KERNEL_CELLWARP) {
+        const int m = (int)std::min<int64_t>(n, kLaunchSteps);
+        const int e = dispatch_prec(s.p.precision, [&](auto P) {
+            return Launch<decltype(P)::value>::steps_cellwarp(s, s.cur, m);
+        });
+        if (e == (int)cudaErrorNotSupported) break;
+        CU(e);
+        s.cur ^= m & 1;
+        s.steps += m;
+        n -= m;
+    }
     if (n >= 2 * kGraphSteps) {
         if ((rc = ensure_step_graph(s, kern))) return rc;
         if (s.cur == 1) { if ((rc = one())) return rc; --n; }

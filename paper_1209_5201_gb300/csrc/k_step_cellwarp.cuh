@@ -1,13 +1,11 @@
 // One-warp-per-cell form of the time step (Eq. (5) with the Eq. (12) wall),
-// for grids of a few thousand cells, where the one-thread-per-cell kernel is
-// bound by the latency of one thread's dependent chain (in FP64 on GB300 each
-// warp instruction of that chain costs the FP64 unit's full issue time).
+// for FP32 and BF16 grids of a few thousand cells, where the one-thread-per-cell
+// kernel is bound by the latency of one thread's dependent chain (FP64 grids:
+// k_step_cellwarp64.cuh).
 //
 // Lane l carries velocities l and l + 32 (Q <= 37): it pulls them, the warp
 // sums the moments with a butterfly of shuffles (every lane gets the totals),
-// every lane forms the shell-independent Eq. (4) factors (FP64: lane s the
-// coefficients of shell s, shuffled to the lanes that need them) and relaxes
-// its own velocities.  Steps are launched with programmatic dependent launch.
+// every lane forms the Eq. (4) coefficients and relaxes its own velocities.  Steps are launched with programmatic dependent launch.
 // A wall row's warp first sums the incoming mass of the ghost columns its
 // fills come from, one term per lane (the wall's term list, <= 26 terms).
 // The moments are summed in another order than the one-thread kernels use,
@@ -35,6 +33,7 @@ k_step_cellwarp(const typename Store<PREC>::S *__restrict__ fin,
     using S = typename Store<PREC>::S;
     using C = typename Store<PREC>::C;
     constexpr bool SHIFT = Store<PREC>::shifted;
+    static_assert(sizeof(C) == 4, "FP64 grids take k_step_cellwarp64");
     // the lattice tables in shared memory, written with compile-time indices
     __shared__ int s_ex[Q], s_ey[Q], s_sh[Q];
     __shared__ int s_tb[2][32], s_tk[2][32];
@@ -144,38 +143,18 @@ k_step_cellwarp(const typename Store<PREC>::S *__restrict__ fin,
     col.set_omega(om);
     col.sx = k.r * ux;
     col.sy = k.r * uy;
-    // Eq. (4) coefficients: the c2-independent factors in every lane, those
-    // of shell s in lane s only (the per-shell work is not repeated by every
-    // lane, which matters where FP64 instructions are slow); each lane then
-    // takes its velocities' shells' values by shuffle
-    // (FP64 only: in FP32 the replicated per-shell work is cheaper than the
-    // shuffles, measured)
+    // Eq. (4) coefficients of every shell in every lane (cheaper than sharing
+    // the per-shell work by shuffles, measured)
     const int sh0 = a0 < Q ? s_sh[a0] : 0, sh1 = a1 < Q ? s_sh[a1] : 0;
     C A0v[2], A1v[2], A2v[2], cwv[2];
-    if constexpr (sizeof(C) == 8) {
-        C pw[8];
-        col.powers(u2, th, drho * inv, k, pw);
-        C sA0 = 0, sA1 = 0, sA2 = 0, scw = 0;
-        if (lane < Lat<Q>::NSH)
-            Collision<Q, C, SHIFT>::shell(pw, om * col.rho, k, lane, sA0, sA1, sA2, scw);
-        const int shv[2] = {sh0, sh1};
+    col.set_coefficients(u2, th, om * col.rho, drho * inv, k);
+    const int shv[2] = {sh0, sh1};
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            A0v[i] = __shfl_sync(0xffffffffu, sA0, shv[i]);
-            A1v[i] = __shfl_sync(0xffffffffu, sA1, shv[i]);
-            A2v[i] = __shfl_sync(0xffffffffu, sA2, shv[i]);
-            cwv[i] = __shfl_sync(0xffffffffu, scw, shv[i]);
-        }
-    } else {
-        col.set_coefficients(u2, th, om * col.rho, drho * inv, k);
-        const int shv[2] = {sh0, sh1};
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            A0v[i] = col.A0[shv[i]];
-            A1v[i] = col.A1[shv[i]];
-            A2v[i] = col.A2[shv[i]];
-            cwv[i] = col.cw[shv[i]];
-        }
+    for (int i = 0; i < 2; ++i) {
+        A0v[i] = col.A0[shv[i]];
+        A1v[i] = col.A1[shv[i]];
+        A2v[i] = col.A2[shv[i]];
+        cwv[i] = col.cw[shv[i]];
     }
 
     // relax and store this lane's velocities (Eq. (4)-(5)); i: 0 for a0, 1 for a1

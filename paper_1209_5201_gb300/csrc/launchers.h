@@ -12,6 +12,8 @@ struct Launch {
     static int direct_variants();
     static int step_staged(SolverImpl &s, int src, int dst, int variant);
     static int step_cellwarp(SolverImpl &s, int src, int dst);
+    // n steps in one launch; cudaErrorNotSupported: use step_cellwarp
+    static int steps_cellwarp(SolverImpl &s, int src, int n);
     static int staged_variants();
     static int init_rest(SolverImpl &s);
     static int init_fields(SolverImpl &s, const double *rho, const double *ux,

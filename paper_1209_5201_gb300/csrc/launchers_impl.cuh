@@ -4,6 +4,7 @@
 #include "k_aux.cuh"
 #include "k_fluxes.cuh"
 #include "k_step_cellwarp.cuh"
+#include "k_step_cellwarp64.cuh"
 #include "k_step_direct.cuh"
 #include "k_step_staged.cuh"
 #include "launchers.h"
@@ -138,11 +139,88 @@ int Launch<PREC>::step_cellwarp(SolverImpl &s, int src, int dst) {
     cfg.numAttrs = 1;
     const S *fin = (const S *)s.f[src];
     S *fout = (S *)s.f[dst];
-    const float *rin = s.rho[src];
-    float *rout = s.rho[dst];
-    LBM_DISPATCH_Q(s.L.Q, return (int)cudaLaunchKernelEx(&cfg, k_step_cellwarp<QQ, PREC>, fin, fout,
-                                                          rin, rout, k));
+    if constexpr (PREC == LBM_FP64) {
+        cfg.gridDim = dim3((unsigned)((cells + kCellWarps - 1) / kCellWarps));
+        cfg.blockDim = dim3(32 * kCellWarps);
+        LBM_DISPATCH_Q(s.L.Q, return (int)cudaLaunchKernelEx(&cfg, k_step_cellwarp64<QQ>, fin, fout,
+                                                              k, s.lanes));
+    } else {
+        const float *rin = s.rho[src];
+        float *rout = s.rho[dst];
+        LBM_DISPATCH_Q(s.L.Q, return (int)cudaLaunchKernelEx(&cfg, k_step_cellwarp<QQ, PREC>, fin,
+                                                              fout, rin, rout, k));
+    }
     return (int)cudaErrorInvalidValue;
+}
+
+// n steps of the one-warp-per-cell kernel from buffer src in one launch, or
+// cudaErrorNotSupported where a launch per step it is: FP32 / BF16 storage, or
+// more cells than resident warps.  Up to 64 cells run on one 16-CTA cluster
+// (one cell per SM sub-partition: the FP64 chain of one cell is then a step's
+// length, and the cluster barrier and a read of distributed shared memory are
+// cheaper than the grid barrier and L2); more cells would queue on the
+// cluster's FP64 units, so they spread over every SM.
+template <int PREC>
+int Launch<PREC>::steps_cellwarp(SolverImpl &s, int src, int n) {
+    if constexpr (PREC != LBM_FP64) {
+        return (int)cudaErrorNotSupported;
+    } else {
+        const long long cells = (long long)s.p.Nx * s.p.Ny;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        cfg.stream = s.stream;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        const double *fin = (const double *)s.f[src];
+        double *fout = (double *)s.f[src ^ (n & 1)];
+        if (cells <= kCellClusterCells && s.cell_cluster >= 0) {
+            unsigned cl = 1;
+            while (cl * kCellWarps < cells) cl *= 2;
+            cfg.gridDim = dim3(cl);
+            cfg.blockDim = dim3(32 * kCellWarps);
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = cl;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            LBM_DISPATCH_Q(s.L.Q, {
+                auto kern = k_steps_cellwarp64_cluster<QQ>;
+                if (s.cell_cluster == 0) {       // once per solver: does it schedule here?
+                    cudaError_t e = cudaFuncSetAttribute(
+                        kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+                    int fit = 0;
+                    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&fit, kern, &cfg);
+                    s.cell_cluster = e == cudaSuccess && fit >= 1 ? 1 : -1;
+                    cudaGetLastError();          // not an error of the caller's
+                }
+                if (s.cell_cluster > 0)
+                    return (int)cudaLaunchKernelEx(&cfg, kern, fin, fout, s.kd, s.lanes, n);
+            });
+        }
+        const long long sms = s.sm_count;
+        int warps = kCellWarps;              // per block: one block per SM
+        while (warps * sms < cells) warps += kCellWarps;
+        if (warps > kCellMaxWarps) return (int)cudaErrorNotSupported;
+        cfg.gridDim = dim3((unsigned)((cells + warps - 1) / warps));
+        cfg.blockDim = dim3(32 * warps);
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+        double *f0 = (double *)s.f[src], *f1 = (double *)s.f[src ^ 1];
+        unsigned *bar = s.bar;
+        int *err = s.derr;
+        LBM_DISPATCH_Q(s.L.Q, {
+            cudaError_t e =
+                warps == kCellWarps
+                    ? cudaLaunchKernelEx(&cfg, k_steps_cellwarp64_grid<QQ, kCellWarps>, f0, f1, s.kd,
+                                         s.lanes, n, bar, err)
+                    : cudaLaunchKernelEx(&cfg, k_steps_cellwarp64_grid<QQ, kCellMaxWarps>, f0, f1,
+                                         s.kd, s.lanes, n, bar, err);
+            if (e == cudaErrorCooperativeLaunchTooLarge) {
+                cudaGetLastError();          // fewer SMs than the device has: a launch per step
+                e = cudaErrorNotSupported;
+            }
+            return (int)e;
+        });
+        return (int)cudaErrorInvalidValue;
+    }
 }
 
 // ---- TMA-staged kernel variants (tile TX x TY, ring of STAGES, CPT cells per

@@ -110,10 +110,29 @@ struct KConsts {
     unsigned long long wait_ns;
 };
 
+// Constants of the FP64 one-warp-per-cell step by lane (k_step_cellwarp64.cuh):
+// lane 0 the rest velocity, lane p the pair (2p - 1, 2p), whose first member's
+// velocity is (ex, ey).
+constexpr int kMaxPairs = (kMaxQ - 1) / 2 + 1;
+struct CellLanes {
+    double cx[kMaxPairs], cy[kMaxPairs];      // r e
+    double x0[kMaxPairs], x1[kMaxPairs], x2[kMaxPairs];   // theta, theta u^2, theta^2 factors of 2 A0
+    double t1[kMaxPairs], t2[kMaxPairs];      // theta factors of A1 and 2 A2
+    double we[kMaxPairs], wo[kMaxPairs];      // w / 2 (of 2E) and w (of O)
+    double mom[4][40];                        // 1, c_x, c_y, |c|^2 / 2 by velocity, zero past Q
+    double tau_half;                          // tau / dt + 1/2 of a constant tau
+    signed char ex[kMaxPairs], ey[kMaxPairs];
+    // incoming terms of each wall (Sec. III): velocity, row from the wall, e_x
+    signed char tb[2][32], tk[2][32], tx[2][32];
+    int nterm;
+    int diffuse[2];                           // accommodation 1
+};
+
 // Kernel constants of one solve (Eq. (4)-(5) factors, Eq. (11)-(12) wall
 // coefficients); defined in api.cpp.
 template <class C>
 void fill_consts(KConsts<C> &k, const LatticeHost &L, const lbm_params &p, int pitch);
+void fill_cell_lanes(CellLanes &c, const LatticeHost &L, const lbm_params &p);
 
 struct SolverImpl {
     LatticeHost L;
@@ -140,9 +159,12 @@ struct SolverImpl {
     double wall_in[2];
     KConsts<float> kf;
     KConsts<double> kd;
+    CellLanes lanes;
+    int cell_cluster;         // many-step launch on one cluster: 0 not asked yet, 1 schedulable, -1 not
     int sm_count;
     int *derr;                // device error flags of the staged kernel
     unsigned *sr;             // step counters of the stochastic BF16 rounding (2)
+    unsigned *bar;            // grid barrier of the many-step cell-warp launch (3 words, zero between)
     int variant;              // staged-kernel variant in use (see launchers)
     long long tm_key;         // (TX, TY) the tensor maps were encoded for; -1 none
     CUtensorMap tm_f[2];      // 3-D maps (x, y, a) of the two state buffers
@@ -152,6 +174,7 @@ struct SolverImpl {
     int graph_kernel, graph_variant;
 };
 
+constexpr int kLaunchSteps = 2048;   // most steps of one many-step launch (a few to 20 ms)
 constexpr int kGraphSteps = 64;   // steps per replayed graph (even: parity kept)
 
 // Encode tm_f / tm_r for boxes of (TX + 2 kPadL) x TY (density: TY + 6 rows).

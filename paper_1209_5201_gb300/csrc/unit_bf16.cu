@@ -5,6 +5,7 @@
 namespace lbm {
 template int Launch<LBM_BF16DEV>::step_staged(SolverImpl &, int, int, int);
 template int Launch<LBM_BF16DEV>::step_cellwarp(SolverImpl &, int, int);
+template int Launch<LBM_BF16DEV>::steps_cellwarp(SolverImpl &, int, int);
 template int Launch<LBM_BF16DEV>::staged_variants();
 template int Launch<LBM_BF16DEV>::init_rest(SolverImpl &);
 template int Launch<LBM_BF16DEV>::init_fields(SolverImpl &, const double *, const double *,

@@ -5,6 +5,7 @@
 namespace lbm {
 template int Launch<LBM_BF16SHIFT>::step_staged(SolverImpl &, int, int, int);
 template int Launch<LBM_BF16SHIFT>::step_cellwarp(SolverImpl &, int, int);
+template int Launch<LBM_BF16SHIFT>::steps_cellwarp(SolverImpl &, int, int);
 template int Launch<LBM_BF16SHIFT>::staged_variants();
 template int Launch<LBM_BF16SHIFT>::init_rest(SolverImpl &);
 template int Launch<LBM_BF16SHIFT>::init_fields(SolverImpl &, const double *, const double *,

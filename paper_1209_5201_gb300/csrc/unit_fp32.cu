@@ -5,6 +5,7 @@
 namespace lbm {
 template int Launch<LBM_FP32>::step_staged(SolverImpl &, int, int, int);
 template int Launch<LBM_FP32>::step_cellwarp(SolverImpl &, int, int);
+template int Launch<LBM_FP32>::steps_cellwarp(SolverImpl &, int, int);
 template int Launch<LBM_FP32>::staged_variants();
 template int Launch<LBM_FP32>::init_rest(SolverImpl &);
 template int Launch<LBM_FP32>::init_fields(SolverImpl &, const double *, const double *,

@@ -5,6 +5,7 @@
 namespace lbm {
 template int Launch<LBM_FP64>::step_staged(SolverImpl &, int, int, int);
 template int Launch<LBM_FP64>::step_cellwarp(SolverImpl &, int, int);
+template int Launch<LBM_FP64>::steps_cellwarp(SolverImpl &, int, int);
 template int Launch<LBM_FP64>::staged_variants();
 template int Launch<LBM_FP64>::init_rest(SolverImpl &);
 template int Launch<LBM_FP64>::init_fields(SolverImpl &, const double *, const double *,
