@@ -267,6 +267,32 @@ void fill_consts(KConsts<C> &k, const LatticeHost &L, const lbm_params &p, int p
     }
 }
 
+void fill_wall(KWall &kw, const LatticeHost &L, const lbm_params &p, const KConsts<float> &k) {
+    std::memset(&kw, 0, sizeof(kw));
+    const bool shifted = p.precision == LBM_FP32 || p.precision == LBM_BF16SHIFT;
+    for (int a = 0; a < L.Q && shifted; ++a)
+        for (int kk = 0; kk < std::abs(L.ey[a]); ++kk) kw.wsum[L.ey[a] < 0 ? 0 : 1] += (double)k.w[a];
+    int nout = 0;
+    for (int a = 1; a < L.Q; ++a)            // opposite pairs are (1, 2), (3, 4), ...
+        if (L.ey[a] > 0) {
+            kw.out_a[0][nout] = (signed char)a;
+            kw.out_a[1][nout++] = (signed char)(a % 2 ? a + 1 : a - 1);
+        }
+    for (int w = 0; w < 2; ++w) {
+        kw.diffuse[w] = p.accom[w] == 1.0;
+        for (int l = 0; l < nout; ++l) {
+            const int a = kw.out_a[w][l];
+            const double c = k.wcoef[w][a];
+            const double c0 = shifted ? std::fma(kw.wsum[w], c, -(double)k.w[a]) : 0.0;
+            KWall::Emit &e = kw.e[w][l];
+            e.ch = (float)c;
+            e.cl = (float)(c - (double)e.ch);
+            e.c0h = (float)c0;
+            e.c0l = (float)(c0 - (double)e.c0h);
+        }
+    }
+}
+
 void fill_cell_lanes(CellLanes &c, const LatticeHost &L, const lbm_params &p) {
     std::memset(&c, 0, sizeof(c));
     for (int l = 0; l <= (L.Q - 1) / 2; ++l) {
@@ -535,6 +561,7 @@ int lbm_solver_create(const lbm_lattice *lat, const lbm_params *p, void *stream,
     }
     fill_consts(s.kd, s.L, s.p, s.pitch);
     fill_consts(s.kf, s.L, s.p, s.pitch);
+    fill_wall(s.kw, s.L, s.p, s.kf);
     fill_cell_lanes(s.lanes, s.L, s.p);
     s.kd.f0 = s.kf.f0 = s.f[0];
     s.kd.sr = s.kf.sr = s.sr;

@@ -21,18 +21,18 @@ template <int Q, int PREC>
 __global__ void __launch_bounds__(kFluxThreads)
 k_fluxes(const typename Store<PREC>::S *__restrict__ fin, const float *__restrict__ rin,
          const __grid_constant__ KConsts<typename Store<PREC>::C> k,
-         const __grid_constant__ KConsts<double> kd, double *sxx, double *sxy, double *syy,
+         const __grid_constant__ KWall kw, const __grid_constant__ KConsts<double> kd, double *sxx, double *sxy, double *syy,
          double *qx, double *qy) {
     using L = Lat<Q>;
     using C = typename Store<PREC>::C;
-    __shared__ double s_min[kFluxThreads + 6];
+    __shared__ WallFills<PREC, kFluxThreads> s_fill;
     const int j = blockIdx.y;
     const int x0 = blockIdx.x * kFluxThreads;
     const int x = x0 + threadIdx.x;
     const bool bot = j < L::N, top = j >= k.Ny - L::N;
     if (bot || top) {
-        wall_prologue<Q, PREC, kFluxThreads>(fin, rin, k, bot ? 0 : 1, x0,
-                                             min(kFluxThreads, k.Nx - x0) + 6, s_min);
+        wall_prologue<Q, PREC, kFluxThreads>(fin, rin, k, kw, bot ? 0 : 1, x0,
+                                             min(kFluxThreads, k.Nx - x0) + 6, s_fill);
         __syncthreads();
     }
     if (x >= k.Nx) return;
@@ -40,8 +40,8 @@ k_fluxes(const typename Store<PREC>::S *__restrict__ fin, const float *__restric
     C fc[Q];
     const typename Store<PREC>::S *src = fin + col_index(k, j, x);
     const float *rsrc = Store<PREC>::dev ? rin + rho_index(k, j, x) : nullptr;
-    if (bot || top) pull<Q, PREC, true, 0>(fin, rin, src, rsrc, k, x, j, s_min, fc);
-    else pull<Q, PREC, false, 0>(fin, rin, src, rsrc, k, x, j, s_min, fc);
+    if (bot || top) pull<Q, PREC, kFluxThreads, true, 0>(fin, rin, src, rsrc, k, kw, x, j, s_fill, fc);
+    else pull<Q, PREC, kFluxThreads, false, 0>(fin, rin, src, rsrc, k, kw, x, j, s_fill, fc);
 
     double f[Q];
     double rho = 0.0, jx = 0.0, jy = 0.0;

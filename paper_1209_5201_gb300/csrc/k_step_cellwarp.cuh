@@ -28,7 +28,8 @@ __global__ void __launch_bounds__(32)
 k_step_cellwarp(const typename Store<PREC>::S *__restrict__ fin,
                 typename Store<PREC>::S *__restrict__ fout, const float *__restrict__ rin,
                 float *__restrict__ rout,
-                const __grid_constant__ KConsts<typename Store<PREC>::C> k) {
+                const __grid_constant__ KConsts<typename Store<PREC>::C> k,
+                const __grid_constant__ KWall kw) {
     using L = Lat<Q>;
     using S = typename Store<PREC>::S;
     using C = typename Store<PREC>::C;
@@ -103,8 +104,9 @@ k_step_cellwarp(const typename Store<PREC>::S *__restrict__ fin,
         const int ex = s_ex[a], sj = j - s_ey[a];
         if (sj < 0 || sj >= k.Ny) {
             const int wall = sj < 0 ? 0 : 1;
-            const C spec = k.accom[wall] != 1.0 ? specular_source<PREC>(fin, rin, k, a, ex, x, j) : C(0);
-            return wall_mix<PREC>(s_min[3 - ex], k.wcoef[wall][a], k.w[a], k.accom[wall], spec);
+            const C v = wall_fill<PREC>(s_min[3 - ex], k.wcoef[wall][a], k.w[a]);
+            if (kw.diffuse[wall]) return v;
+            return wall_mix<PREC>(v, k.accom[wall], specular_source<PREC>(fin, rin, k, a, ex, x, j));
         }
         return load(a, sj, wrap(x - ex, k.Nx));
     };

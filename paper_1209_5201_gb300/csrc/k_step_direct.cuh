@@ -13,7 +13,7 @@
 // instructions; otherwise they are per-velocity byte offsets added to the
 // cell's address.  Blocks holding any of the N rows next to a wall first sum
 // that wall's incoming mass M_in for the BX + 6 ghost columns their fill
-// populations come from (FP64, fixed order).
+// populations come from (fixed order, to FP64 precision).
 #pragma once
 
 #include <type_traits>
@@ -22,60 +22,42 @@
 
 namespace lbm {
 
-// M_in(x') for x' = x0 - 3 + t, t in [0, ncols): post-collision populations
-// of the N rows next to `wall` that stream into ghost column x' (Sec. III:
-// incoming at layer l when e.n < -l; summed over all layers, Eq. (12)).
+// Re-emissions of the ghost columns x0 - 3 + t, t in [0, ncols), one column
+// per thread: s_fill[l][t] for the l-th outgoing velocity.
+template <int PREC, int BX>
+using WallFills = typename Store<PREC>::C[kMaxWallOut][BX + 6];
 template <int Q, int PREC, int BX>
 __device__ __forceinline__ void wall_prologue(const typename Store<PREC>::S *__restrict__ fin,
                                               const float *__restrict__ rin,
                                               const KConsts<typename Store<PREC>::C> &k,
-                                              int wall, int x0, int ncols, double *s_min) {
-    using L = Lat<Q>;
-    for (int t = threadIdx.x; t < ncols; t += BX) {
-        const int xw = wrap(x0 - 3 + t, k.Nx);
-        double m = 0.0;
-#pragma unroll
-        for (int b = 0; b < Q; ++b) {
-            const int eyb = L::ey(b);
-            const bool incoming = wall == 0 ? (eyb < 0) : (eyb > 0);
-            if (!incoming) continue;
-            const int xs = wrap(xw - L::ex(b), k.Nx);
-            const int depth = eyb < 0 ? -eyb : eyb;
-            for (int kk = 0; kk < depth; ++kk) {
-                const int row = wall == 0 ? kk : k.Ny - 1 - kk;
-                double v = (double)to_c(fin[col_index(k, row, xs) + (long long)b * k.pitch]);
-                if constexpr (Store<PREC>::dev)
-                    v += (double)k.w[b] * (double)rin[rho_index(k, row, xs)];
-                if constexpr (Store<PREC>::shifted) v += (double)k.w[b];
-                m += v;
-            }
-        }
-        s_min[t] = m;
-    }
+                                              const KWall &kw, int wall, int x0, int ncols,
+                                              WallFills<PREC, BX> &s_fill) {
+    for (int t = threadIdx.x; t < ncols; t += BX)
+        wall_column_fill<Q, PREC>(fin, rin, k, kw, wall, x0 - 3 + t, &s_fill[0][t], BX + 6);
 }
 
 // Pull of cell (x, j): src is the cell's own element (velocity 0) in its
 // tile, rsrc its density (BF16DEV).  PC > 0: the tile pitch, a compile-time
 // constant; PC = 0: the solver's pitch, offsets from the constants.
-template <int Q, int PREC, bool WALL, int PC>
+template <int Q, int PREC, int BX, bool WALL, int PC>
 __device__ __forceinline__ void pull(const typename Store<PREC>::S *__restrict__ fin,
                                      const float *__restrict__ rin,
                                      const typename Store<PREC>::S *__restrict__ src,
                                      const float *__restrict__ rsrc,
-                                     const KConsts<typename Store<PREC>::C> &k, int x, int j,
-                                     const double *s_min, typename Store<PREC>::C (&f)[Q]) {
+                                     const KConsts<typename Store<PREC>::C> &k, const KWall &kw,
+                                     int x, int j, const WallFills<PREC, BX> &s_fill,
+                                     typename Store<PREC>::C (&f)[Q]) {
     using L = Lat<Q>;
     using S = typename Store<PREC>::S;
     using C = typename Store<PREC>::C;
     StaticFor<0, Q>::run([&](auto ac) {
         constexpr int a = decltype(ac)::value;
         const int sj = j - L::ey(a);
-        if (WALL && (sj < 0 || sj >= k.Ny)) {
-            const int wall = sj < 0 ? 0 : 1;
-            const C spec = k.accom[wall] != 1.0
-                               ? specular_source<PREC>(fin, rin, k, a, L::ex(a), x, j) : C(0);
-            f[a] = wall_mix<PREC>(s_min[threadIdx.x + 3 - L::ex(a)], k.wcoef[wall][a], k.w[a],
-                                  k.accom[wall], spec);
+        bool wall_src = false;
+        if constexpr (WALL && L::ey(a) > 0) wall_src = sj < 0;
+        if constexpr (WALL && L::ey(a) < 0) wall_src = sj >= k.Ny;
+        if (wall_src) {
+            f[a] = s_fill[L::out_rank(a)][(int)threadIdx.x + 3 - L::ex(a)];
         } else {
             C v;
             if constexpr (PC > 0) {
@@ -92,6 +74,16 @@ __device__ __forceinline__ void pull(const typename Store<PREC>::S *__restrict__
             f[a] = v;
         }
     });
+    if (WALL && !kw.diffuse[j < L::N ? 0 : 1]) {
+        const int wall = j < L::N ? 0 : 1;
+        StaticFor<0, Q>::run([&](auto ac) {
+            constexpr int a = decltype(ac)::value;
+            const int sj = j - L::ey(a);
+            if (sj < 0 || sj >= k.Ny)
+                f[a] = wall_mix<PREC>(f[a], k.accom[wall],
+                                      specular_source<PREC>(fin, rin, k, a, L::ex(a), x, j));
+        });
+    }
 }
 
 // Store of population A of the cell whose own element is dst (velocity 0).
@@ -108,6 +100,58 @@ __device__ __forceinline__ void store_one(S *dst, const KConsts<C> &k, S v) {
             st_b<CS>(reinterpret_cast<unsigned short *>(dst), k.b_dst[A], __bfloat16_as_ushort(v));
         else
             st_b<CS>(dst, k.b_dst[A], v);
+    }
+}
+
+// Store of a cell's Q values v (BF16DEV: and its density) in its own slots
+// (dst: its element of velocity 0; rdst: its density) and, for the kPadL
+// columns at either end of tile t (xl of w columns), the halo copies.  All
+// values first, the copies behind one branch: a branch per velocity between
+// the stores costs the 4096 x 2048 FP32 step 17 %.
+template <int Q, int PREC, bool CS, int PC>
+__device__ __forceinline__ void store_cell(const typename Store<PREC>::S (&v)[Q], float rho,
+                                           typename Store<PREC>::S *__restrict__ fout,
+                                           float *__restrict__ rout,
+                                           typename Store<PREC>::S *__restrict__ dst,
+                                           float *__restrict__ rdst,
+                                           const KConsts<typename Store<PREC>::C> &k, int t, int xl,
+                                           int w, int j) {
+    using S = typename Store<PREC>::S;
+    StaticFor<0, Q>::run([&](auto ac) {
+        constexpr int A = decltype(ac)::value;
+        store_one<PC, CS, A>(dst, k, v[A]);
+    });
+    if constexpr (Store<PREC>::dev) *rdst = rho;
+    if (xl < kPadL || xl >= w - kPadL) {
+        if (w >= 2 * kPadL) {
+            // one copy, at the same offset from every velocity's slot: in the
+            // previous tile's right halo (xl < kPadL) or the next tile's left
+            // halo (with one tile: the periodic image x + Nx or x - Nx)
+            long long d, dr;
+            if (xl < kPadL) {
+                const int tl = t == 0 ? k.nt - 1 : t - 1;
+                const int wl = tile_width(k, tl);
+                d = (tl - t) * k.tile_elems + wl;
+                dr = (tl - t) * k.tile_rho + wl;
+            } else {
+                const int tr = t == k.nt - 1 ? 0 : t + 1;
+                d = (tr - t) * k.tile_elems - w;
+                dr = (tr - t) * k.tile_rho - w;
+            }
+            StaticFor<0, Q>::run([&](auto ac) {
+                constexpr int A = decltype(ac)::value;
+                store_one<PC, CS, A>(dst + d, k, v[A]);
+            });
+            if constexpr (Store<PREC>::dev) rdst[dr] = rho;
+        } else {
+            // a grid narrower than 2 kPadL: several images per column
+            const long long rowq = (long long)j * k.Q;
+#pragma unroll
+            for (int a = 0; a < Q; ++a)
+                store_halo_copies<S>(fout + (rowq + a) * k.pitch, k.tile_elems, k, t, xl, w, v[a]);
+            if constexpr (Store<PREC>::dev)
+                store_halo_copies<float>(rout + (long long)j * k.pitch, k.tile_rho, k, t, xl, w, rho);
+        }
     }
 }
 
@@ -159,43 +203,7 @@ __device__ __forceinline__ void collide_store(const typename Store<PREC>::C (&f)
 #pragma unroll
         for (int a = 0; a < Q; ++a) v[a] = store_rounded<S>(o[a], 0u);
     }
-    StaticFor<0, Q>::run([&](auto ac) {
-        constexpr int A = decltype(ac)::value;
-        store_one<PC, CS, A>(dst, k, v[A]);
-    });
-    if constexpr (Store<PREC>::dev) *rdst = (float)col.rho;
-    if (xl < kPadL || xl >= w - kPadL) {
-        if (w >= 2 * kPadL) {
-            // one copy, at the same offset from every velocity's slot: in the
-            // previous tile's right halo (xl < kPadL) or the next tile's left
-            // halo (with one tile: the periodic image x + Nx or x - Nx)
-            long long d, dr;
-            if (xl < kPadL) {
-                const int tl = t == 0 ? k.nt - 1 : t - 1;
-                const int wl = tile_width(k, tl);
-                d = (tl - t) * k.tile_elems + wl;
-                dr = (tl - t) * k.tile_rho + wl;
-            } else {
-                const int tr = t == k.nt - 1 ? 0 : t + 1;
-                d = (tr - t) * k.tile_elems - w;
-                dr = (tr - t) * k.tile_rho - w;
-            }
-            StaticFor<0, Q>::run([&](auto ac) {
-                constexpr int A = decltype(ac)::value;
-                store_one<PC, CS, A>(dst + d, k, v[A]);
-            });
-            if constexpr (Store<PREC>::dev) rdst[dr] = (float)col.rho;
-        } else {
-            // a grid narrower than 2 kPadL: several images per column
-            const long long rowq = (long long)j * k.Q;
-#pragma unroll
-            for (int a = 0; a < Q; ++a)
-                store_halo_copies<S>(fout + (rowq + a) * k.pitch, k.tile_elems, k, t, xl, w, v[a]);
-            if constexpr (Store<PREC>::dev)
-                store_halo_copies<float>(rout + (long long)j * k.pitch, k.tile_rho, k, t, xl, w,
-                                         (float)col.rho);
-        }
-    }
+    store_cell<Q, PREC, CS, PC>(v, (float)col.rho, fout, rout, dst, rdst, k, t, xl, w, j);
 }
 
 // BX threads per block (one row segment of a tile); MINB blocks per SM
@@ -208,10 +216,16 @@ __global__ void __launch_bounds__(BX, MINB)
 k_step_direct(const typename Store<PREC>::S *__restrict__ fin,
               typename Store<PREC>::S *__restrict__ fout, const float *__restrict__ rin,
               float *__restrict__ rout,
-              const __grid_constant__ KConsts<typename Store<PREC>::C> k) {
+              const __grid_constant__ KConsts<typename Store<PREC>::C> k,
+              const __grid_constant__ KWall kw) {
     using L = Lat<Q>;
     using C = typename Store<PREC>::C;
-    __shared__ double s_min[2][BX + 6];
+    // both walls' fills only where one block can hold rows of both
+    __shared__ WallFills<PREC, BX> s_fill[RS > 1 ? 2 : 1];
+    // launched with programmatic stream serialization: the next step's blocks
+    // may take the places of finished ones, and everything before the wait
+    // overlaps the previous step's last blocks
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int bpt = (k.tw + BX - 1) / BX;
     const int t = blockIdx.x / bpt, xl0 = (blockIdx.x - t * bpt) * BX;
     const int w = tile_width(k, t);
@@ -221,8 +235,14 @@ k_step_direct(const typename Store<PREC>::S *__restrict__ fin,
     const int j1 = min(k.Ny, j0 + RS);
     const bool bot = j0 < L::N, top = j1 > k.Ny - L::N;
     const int ncols = min(BX, w - xl0) + 6;
-    if (bot) wall_prologue<Q, PREC, BX>(fin, rin, k, 0, t * k.tw + xl0, ncols, s_min[0]);
-    if (top) wall_prologue<Q, PREC, BX>(fin, rin, k, 1, t * k.tw + xl0, ncols, s_min[1]);
+    // the previous step's stores are visible from here on
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    if (RS > 1) {
+        if (bot) wall_prologue<Q, PREC, BX>(fin, rin, k, kw, 0, t * k.tw + xl0, ncols, s_fill[0]);
+        if (top) wall_prologue<Q, PREC, BX>(fin, rin, k, kw, 1, t * k.tw + xl0, ncols, s_fill[RS > 1 ? 1 : 0]);
+    } else if (bot || top) {
+        wall_prologue<Q, PREC, BX>(fin, rin, k, kw, bot ? 0 : 1, t * k.tw + xl0, ncols, s_fill[0]);
+    }
     if (bot || top) __syncthreads();
     // BF16: step count of the stochastic rounding (block 0 advances it)
     uint32_t seed = 0;
@@ -239,10 +259,10 @@ k_step_direct(const typename Store<PREC>::S *__restrict__ fin,
         float *rdst = Store<PREC>::dev ? rout + rcell : nullptr;
         C f[Q];
         if (j < L::N || j >= k.Ny - L::N)
-            pull<Q, PREC, true, PC>(fin, rin, fin + cell, rsrc, k, x, j, s_min[j < L::N ? 0 : 1],
-                                    f);
+            pull<Q, PREC, BX, true, PC>(fin, rin, fin + cell, rsrc, k, kw, x, j,
+                                        s_fill[RS > 1 && j >= L::N ? 1 : 0], f);
         else
-            pull<Q, PREC, false, PC>(fin, rin, fin + cell, rsrc, k, x, j, s_min[0], f);
+            pull<Q, PREC, BX, false, PC>(fin, rin, fin + cell, rsrc, k, kw, x, j, s_fill[0], f);
         collide_store<Q, PREC, CS, PC>(f, fout, rout, fout + cell, rdst, k, t, xl, w, x, j, seed);
     }
 }

@@ -104,8 +104,8 @@ struct StagedCfg {
     static constexpr int kConsumerWarps = kConsumers / 32;
     static constexpr int kThreads = kConsumers + 32;
     // 128 bytes of slack for aligning the dynamic base, 1 KB of barriers,
-    // the stage ring, and the two walls' incoming-mass sums
-    static constexpr int kSmem = 128 + 1024 + STAGES * kStageBytes + 2 * (TX + 6) * 8;
+    // the stage ring, and the two walls' re-emissions
+    static constexpr int kSmem = 128 + 1024 + STAGES * kStageBytes + 2 * kMaxWallOut * (TX + 6) * (int)sizeof(typename Store<PREC>::C);
     static_assert(kSmem <= 227 * 1024, "shared memory per CTA");
     static_assert(kConsumers % 32 == 0, "consumer threads must fill warps");
     static_assert(TX % 32 == 0, "tile width must be a multiple of 32 columns");
@@ -119,20 +119,22 @@ k_step_staged(const __grid_constant__ CUtensorMap tm_f, const __grid_constant__ 
               const typename Store<PREC>::S *__restrict__ fin,
               typename Store<PREC>::S *__restrict__ fout, const float *__restrict__ rin,
               float *__restrict__ rout, int *__restrict__ err,
-              const __grid_constant__ KConsts<typename Store<PREC>::C> k) {
+              const __grid_constant__ KConsts<typename Store<PREC>::C> k,
+              const __grid_constant__ KWall kw) {
     using Cfg = StagedCfg<Q, PREC, TX, TY, STAGES, CPT>;
     using L = Lat<Q>;
     using S = typename Store<PREC>::S;
     using C = typename Store<PREC>::C;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    // 1 KB header: barriers; then the stage ring; then the wall sums
+    // 1 KB header: barriers; then the stage ring; then the wall fills
     unsigned char *base = (unsigned char *)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
     uint64_t *full = (uint64_t *)base;
     uint64_t *empty = full + STAGES;
     uint64_t *wbar = empty + STAGES;        // consumers' barrier around the wall sums
     int *stop = (int *)(wbar + 1);
     unsigned char *ring = base + 1024;
-    double *s_min = (double *)(ring + STAGES * Cfg::kStageBytes);   // [2][TX + 6]
+    // wall fills [2][kMaxWallOut][TX + 6]
+    C *s_fill = (C *)(ring + STAGES * Cfg::kStageBytes);
 
     const int ntx = (k.Nx + TX - 1) / TX;
     const int nty = (k.Ny + TY - 1) / TY;
@@ -201,7 +203,7 @@ k_step_staged(const __grid_constant__ CUtensorMap tm_f, const __grid_constant__ 
         const int x0 = (t % ntx) * TX, j0 = (t / ntx) * TY;
         const bool wb = j0 < L::N, wt = j0 + TY > k.Ny - L::N;
         if (wb || wt) {
-            // Eq. (12) numerator for ghost columns x0 - 3 .. x0 + TX + 2, FP64;
+            // Eq. (12) for ghost columns x0 - 3 .. x0 + TX + 2;
             // the first barrier keeps the previous wall tile's readers safe
             if (!wall_sync()) {
                 atomicOr(err, kStagedErrTimeout);
@@ -210,26 +212,11 @@ k_step_staged(const __grid_constant__ CUtensorMap tm_f, const __grid_constant__ 
             }
             for (int w = 0; w < 2; ++w) {
                 if (!(w == 0 ? wb : wt)) continue;
-                for (int c = tid; c < TX + 6; c += Cfg::kConsumers) {
-                    const int xw = wrap(x0 - 3 + c, k.Nx);
-                    double m = 0.0;
-#pragma unroll
-                    for (int b = 0; b < Q; ++b) {
-                        const int eyb = L::ey(b);
-                        if (w == 0 ? !(eyb < 0) : !(eyb > 0)) continue;
-                        const int xs = wrap(xw - L::ex(b), k.Nx);
-                        const int depth = eyb < 0 ? -eyb : eyb;
-                        for (int kk = 0; kk < depth; ++kk) {
-                            const int row = w == 0 ? kk : k.Ny - 1 - kk;
-                            double v = (double)to_c(
-                                fin[col_index(k, row, xs) + (long long)b * k.pitch]);
-                            if constexpr (Cfg::kDev)
-                                v += (double)k.w[b] * (double)rin[rho_index(k, row, xs)];
-                            if constexpr (Store<PREC>::shifted) v += (double)k.w[b];
-                            m += v;
-                        }
-                    }
-                    s_min[w * (TX + 6) + c] = m;
+                // columns of cells past the grid's edge are not formed (nor used)
+                const int nc = min(TX, k.Nx - x0) + 6;
+                for (int c = tid; c < nc; c += Cfg::kConsumers) {
+                    wall_column_fill<Q, PREC>(fin, rin, k, kw, w, x0 - 3 + c,
+                                              s_fill + w * kMaxWallOut * (TX + 6) + c, TX + 6);
                 }
             }
             if (!wall_sync()) {
@@ -252,16 +239,16 @@ k_step_staged(const __grid_constant__ CUtensorMap tm_f, const __grid_constant__ 
             const int cell = tid + q * Cfg::kConsumers;
             const int i = cell % TX, kr = cell / TX;
             const int j = j0 + kr;
-#pragma unroll
-            for (int a = 0; a < Q; ++a) {
+            StaticFor<0, Q>::run([&](auto ac) {
+                constexpr int a = decltype(ac)::value;
                 const int sj = j - L::ey(a);
                 if ((wb || wt) && (sj < 0 || sj >= k.Ny)) {
                     const int wall = sj < 0 ? 0 : 1;
-                    const C spec = (k.accom[wall] != 1.0 && x0 + i < k.Nx && j < k.Ny)
-                                       ? specular_source<PREC>(fin, rin, k, a, L::ex(a), x0 + i, j)
-                                       : C(0);
-                    fv[q][a] = wall_mix<PREC>(s_min[wall * (TX + 6) + i + 3 - L::ex(a)],
-                                              k.wcoef[wall][a], k.w[a], k.accom[wall], spec);
+                    fv[q][a] = s_fill[(wall * kMaxWallOut + L::out_rank(a)) * (TX + 6) + i + 3 - L::ex(a)];
+                    if (!kw.diffuse[wall] && x0 + i < k.Nx && j < k.Ny)
+                        fv[q][a] = wall_mix<PREC>(
+                            fv[q][a], k.accom[wall],
+                            specular_source<PREC>(fin, rin, k, a, L::ex(a), x0 + i, j));
                 } else {
                     const S *pl = (const S *)(st + a * Cfg::kPlaneStride);
                     C v = to_c(pl[kr * Cfg::kW + i + kPadL - L::ex(a)]);
@@ -269,7 +256,7 @@ k_step_staged(const __grid_constant__ CUtensorMap tm_f, const __grid_constant__ 
                         v = dev_to_f(v, k.w[a], srho[(kr + 3 - L::ey(a)) * Cfg::kW + i + kPadL - L::ex(a)]);
                     fv[q][a] = v;
                 }
-            }
+            });
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);

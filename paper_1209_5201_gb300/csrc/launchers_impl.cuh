@@ -53,31 +53,36 @@ int launch_direct(SolverImpl &s, int src, int dst) {
     using S = typename Store<PREC>::S;
     const auto &k = Consts<PREC>::get(s);
     // blocks of BX columns never straddle two x-tiles
-    dim3 grid(k.nt * ((k.tw + BX - 1) / BX), (s.p.Ny + RS - 1) / RS);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(k.nt * ((k.tw + BX - 1) / BX), (s.p.Ny + RS - 1) / RS);
+    cfg.blockDim = dim3(BX);
+    cfg.stream = s.stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const S *fin = (const S *)s.f[src];
+    S *fout = (S *)s.f[dst];
+    const float *rin = s.rho[src];
+    float *rout = s.rho[dst];
     // a pitch class: offsets as instruction immediates (compiled for the
     // 37-velocity lattice; the others take the offsets from the constants)
     if constexpr (Q == 37 && BX == 128 && RS == 1) {
         constexpr int P0 = pitch_class(PREC, 0), P1 = pitch_class(PREC, 1),
                       P2 = pitch_class(PREC, 2);
-        if (k.pitch == P0) {
-            k_step_direct<Q, PREC, BX, MINB, CS, RS, P0><<<grid, BX, 0, s.stream>>>(
-                (const S *)s.f[src], (S *)s.f[dst], s.rho[src], s.rho[dst], k);
-            return (int)cudaGetLastError();
-        }
-        if (k.pitch == P1) {
-            k_step_direct<Q, PREC, BX, MINB, CS, RS, P1><<<grid, BX, 0, s.stream>>>(
-                (const S *)s.f[src], (S *)s.f[dst], s.rho[src], s.rho[dst], k);
-            return (int)cudaGetLastError();
-        }
-        if (k.pitch == P2) {
-            k_step_direct<Q, PREC, BX, MINB, CS, RS, P2><<<grid, BX, 0, s.stream>>>(
-                (const S *)s.f[src], (S *)s.f[dst], s.rho[src], s.rho[dst], k);
-            return (int)cudaGetLastError();
-        }
+        if (k.pitch == P0)
+            return (int)cudaLaunchKernelEx(&cfg, k_step_direct<Q, PREC, BX, MINB, CS, RS, P0>, fin,
+                                           fout, rin, rout, k, s.kw);
+        if (k.pitch == P1)
+            return (int)cudaLaunchKernelEx(&cfg, k_step_direct<Q, PREC, BX, MINB, CS, RS, P1>, fin,
+                                           fout, rin, rout, k, s.kw);
+        if (k.pitch == P2)
+            return (int)cudaLaunchKernelEx(&cfg, k_step_direct<Q, PREC, BX, MINB, CS, RS, P2>, fin,
+                                           fout, rin, rout, k, s.kw);
     }
-    k_step_direct<Q, PREC, BX, MINB, CS, RS, 0><<<grid, BX, 0, s.stream>>>(
-        (const S *)s.f[src], (S *)s.f[dst], s.rho[src], s.rho[dst], k);
-    return (int)cudaGetLastError();
+    return (int)cudaLaunchKernelEx(&cfg, k_step_direct<Q, PREC, BX, MINB, CS, RS, 0>, fin, fout, rin,
+                                   rout, k, s.kw);
 }
 
 // One lattice's direct-kernel variants (the 37-velocity ones, with their
@@ -148,7 +153,7 @@ int Launch<PREC>::step_cellwarp(SolverImpl &s, int src, int dst) {
         const float *rin = s.rho[src];
         float *rout = s.rho[dst];
         LBM_DISPATCH_Q(s.L.Q, return (int)cudaLaunchKernelEx(&cfg, k_step_cellwarp<QQ, PREC>, fin,
-                                                              fout, rin, rout, k));
+                                                              fout, rin, rout, k, s.kw));
     }
     return (int)cudaErrorInvalidValue;
 }
@@ -265,7 +270,7 @@ int launch_staged(SolverImpl &s, int src, int dst) {
     const auto &k = Consts<PREC>::get(s);
     kern<<<grid, Cfg::kThreads, Cfg::kSmem, s.stream>>>(
         s.tm_f[src], s.tm_r[src], (const S *)s.f[src], (S *)s.f[dst], s.rho[src], s.rho[dst],
-        s.derr, k);
+        s.derr, k, s.kw);
     return (int)cudaGetLastError();
 }
 
@@ -354,7 +359,7 @@ int Launch<PREC>::fluxes(SolverImpl &s, double *sxx, double *sxy, double *syy, d
     const auto &k = Consts<PREC>::get(s);
     dim3 grid((s.p.Nx + kFluxThreads - 1) / kFluxThreads, s.p.Ny);
     LBM_DISPATCH_Q(s.L.Q, (k_fluxes<QQ, PREC><<<grid, kFluxThreads, 0, s.stream>>>(
-                               (const S *)s.f[s.cur], s.rho[s.cur], k, s.kd, sxx, sxy, syy, qx,
+                               (const S *)s.f[s.cur], s.rho[s.cur], k, s.kw, s.kd, sxx, sxy, syy, qx,
                                qy)));
     return (int)cudaGetLastError();
 }

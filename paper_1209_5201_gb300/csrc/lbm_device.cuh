@@ -22,6 +22,21 @@ template <int Q> struct Lat;
         __host__ __device__ static constexpr int ey(int a) { constexpr int t[] = EY; return t[a]; } \
         __host__ __device__ static constexpr int sh(int a) { constexpr int t[] = SH; return t[a]; } \
         __host__ __device__ static constexpr int e2(int a) { return ex(a) * ex(a) + ey(a) * ey(a); } \
+        /* opposite velocity, and the rank of velocity a (e_y != 0), or of its   */   \
+        /* opposite, among the velocities with e_y > 0 (KWall::out_a)            */   \
+        __host__ __device__ static constexpr int opp(int a) { return a == 0 ? 0 : (a & 1 ? a + 1 : a - 1); } \
+        __host__ __device__ static constexpr int out_rank(int a) {                    \
+            const int up = ey(a) > 0 ? a : opp(a);                                     \
+            int n = 0;                                                                  \
+            for (int b = 0; b < up; ++b) n += ey(b) > 0 ? 1 : 0;                        \
+            return n;                                                                   \
+        }                                                                               \
+        /* number of velocities with e_y > 0 */                                        \
+        __host__ __device__ static constexpr int nout() {                              \
+            int n = 0;                                                                  \
+            for (int b = 0; b < Q; ++b) n += ey(b) > 0 ? 1 : 0;                         \
+            return n;                                                                   \
+        }                                                                               \
         /* |e|^2 of shell s: that of its first member */                              \
         __host__ __device__ static constexpr int shell_e2(int s) {                     \
             for (int a = 0; a < Q; ++a) if (sh(a) == s) return e2(a);                  \
@@ -604,24 +619,165 @@ __device__ __forceinline__ typename Store<PREC>::C wall_fill(double m_in, double
     return (typename Store<PREC>::C)v;
 }
 
-// Eq. (9) with R = accom R_D + (1 - accom) R_S: the diffuse re-emission mixed
-// with the specular one, `spec` being the mirrored population in the form the
-// collision takes (a deviation for shifted storage; the mirror shares w_a).
+// Eq. (9) with R = accom R_D + (1 - accom) R_S, accom < 1: the diffuse
+// re-emission mixed with the specular one, both in the form the collision
+// takes (a deviation for shifted storage; the mirror shares w_a).
 template <int PREC>
-__device__ __forceinline__ typename Store<PREC>::C wall_mix(double m_in, double coef,
-                                                            typename Store<PREC>::C w,
+__device__ __forceinline__ typename Store<PREC>::C wall_mix(typename Store<PREC>::C diffuse,
                                                             double accom,
                                                             typename Store<PREC>::C spec) {
-    using C = typename Store<PREC>::C;
-    const C diffuse = wall_fill<PREC>(m_in, coef, w);
-    return accom == 1.0 ? diffuse : (C)(accom * (double)diffuse + (1.0 - accom) * (double)spec);
+    return (typename Store<PREC>::C)(accom * (double)diffuse + (1.0 - accom) * (double)spec);
+}
+
+// ---- wall fills of the one-thread-per-cell and tile-staged kernels --------------
+// A block next to a wall first forms, for every ghost column its cells pull
+// from, the incoming mass M_in and from it the re-emission of every outgoing
+// velocity, into shared memory.  Two things bound this on GB300:
+//  * every FP64 warp instruction, conversions and comparisons included, holds
+//    an SM sub-partition's FP64 unit for 64 cycles, and there were about 100
+//    per wall cell (26 terms, 15 re-emissions for D2Q37).  For the FP32 and
+//    BF16 formats the sum runs in FP32 with error-free additions (Knuth's
+//    TwoSum; three floats hold it to far below FP64's rounding) and each
+//    re-emission is evaluated as c0 + d c in pairs of floats with a bound on its
+//    error; only where the bound straddles an FP32 rounding boundary (about one
+//    in 10^5) is it formed again in FP64.  The result is the FP64 expression rounded to FP32;
+//  * instruction fetch: with the re-emission inlined at every velocity of the
+//    pull, twice (two walls), a small grid's wall blocks ran through code they
+//    had no time to cache.  One copy serves both walls (velocity and opposite),
+//    the re-emissions are a loop, the pull reads its fill from shared memory.
+// D2Q37 FP32 on 300 x 40 (a step as long as its wall blocks), us per step: 19.1
+// in FP64; 10.1 in FP32, inlined; 7.8 as a loop; 5.3 with the re-emissions
+// branch-free and the launch overlapped.  4096 x 2048, whose wall blocks end
+// the step: FP32 378 -> 360, BF16SHIFT 262 -> 234; 3001 x 1203 BF16DEV 164 -> 133.
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+    s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+struct Sum3 {                                // a running sum h + m + l
+    float h = 0.0f, m = 0.0f, l = 0.0f;
+    __device__ __forceinline__ void add(float x) {
+        float e, e2;
+        two_sum(h, x, h, e);
+        two_sum(m, e, m, e2);
+        l = __fadd_rn(l, e2);
+    }
+};
+
+// The FP64 expressions of a column's re-emissions, from the sum's three floats.
+// Out of line, so that the compiler does not evaluate them along the FP32 ones.
+template <int Q, int PREC, class K>
+__device__ __noinline__ void wall_fill_exact(float h, float m, float l, const K &k, const KWall &kw,
+                                             int wall, float *out, int stride) {
+    const double m64 = kw.wsum[wall] + ((double)h + ((double)m + (double)l));
+#pragma unroll 1
+    for (int i = 0; i < Lat<Q>::nout(); ++i) {
+        const int a = kw.out_a[wall][i];
+        out[i * stride] = wall_fill<PREC>(m64, k.wcoef[wall][a], k.w[a]);
+    }
+}
+
+// Re-emissions (Eq. (12)) of ghost column xw, -3 <= xw < Nx + 3, of `wall`, in the form the collision takes: out[l * stride] for the l-th
+// outgoing velocity.  M_in sums the post-collision populations of the N rows
+// next to the wall that stream into the column (Sec. III: incoming at layer l
+// when e.n < -l, over all layers).
+template <int Q, int PREC>
+__device__ __forceinline__ void
+wall_column_fill(const typename Store<PREC>::S *__restrict__ fin, const float *__restrict__ rin,
+                 const KConsts<typename Store<PREC>::C> &k, const KWall &kw, int wall, int xw,
+                 typename Store<PREC>::C *out, int stride) {
+    using L = Lat<Q>;
+    // the incoming velocities of wall 0 are those with e_y < 0; wall 1 takes
+    // their opposites, mirrored columns and rows counted from the top.  Elements
+    // of the source columns xw - e_x in row 0 (offsets fit 31 bits)
+    int col[7], rcol[7];
+    const int sgn = wall == 0 ? 1 : -1;
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+        int xs = xw - sgn * (i - 3);
+        if (k.Nx >= 16) xs = xs < 0 ? xs + k.Nx : (xs >= k.Nx ? xs - k.Nx : xs);
+        else xs = wrap(xs, k.Nx);
+        col[i] = xs + kPadL;
+        if constexpr (Store<PREC>::dev) rcol[i] = xs + kPadL;
+    }
+    if (k.nt != 1) {                         // several x-tiles: the element in its tile
+#pragma unroll
+        for (int i = 0; i < 7; ++i) {
+            const int xs = col[i] - kPadL;
+            col[i] = (int)col_index(k, 0, xs);
+            if constexpr (Store<PREC>::dev) rcol[i] = (int)rho_index(k, 0, xs);
+        }
+    }
+    (void)rcol;
+    // rows kk = 0, 1, 2 from the wall; an opposite velocity is one segment
+    // further (odd b) or nearer (even b)
+    const int row0 = wall == 0 ? 0 : k.Ny - 1, pitch = k.pitch, dp = wall == 0 ? 0 : k.pitch;
+    const typename Store<PREC>::S *rows[3];
+    const float *rrows[3] = {nullptr, nullptr, nullptr};
+#pragma unroll
+    for (int kk = 0; kk < 3; ++kk) {
+        rows[kk] = fin + (long long)(row0 + sgn * kk) * Q * pitch;
+        if constexpr (Store<PREC>::dev) rrows[kk] = rin + (long long)(row0 + sgn * kk) * pitch;
+    }
+    (void)rrows;
+    double m64 = 0.0;
+    Sum3 sum;
+    StaticFor<1, Q>::run([&](auto ac) {
+        constexpr int b = decltype(ac)::value;
+        if constexpr (L::ey(b) < 0) {
+#pragma unroll
+            for (int kk = 0; kk < -L::ey(b); ++kk) {
+                const auto v = to_c(rows[kk][b * pitch + (col[L::ex(b) + 3] + (b & 1 ? dp : -dp))]);
+                if constexpr (PREC == LBM_FP64) {
+                    m64 += v;
+                } else {
+                    if constexpr (Store<PREC>::dev) {
+                        // f = d + w rho: the product and its rounding error
+                        const float rho = rrows[kk][rcol[L::ex(b) + 3]];
+                        const float pr = __fmul_rn(k.w[b], rho);
+                        sum.add(__fmaf_rn(k.w[b], rho, -pr));
+                        sum.add(pr);
+                    }
+                    sum.add(v);
+                }
+            }
+        }
+    });
+    if constexpr (PREC == LBM_FP64) {
+#pragma unroll
+        for (int l = 0; l < L::nout(); ++l) {
+            const int a = kw.out_a[wall][l];
+            out[l * stride] = wall_fill<PREC>(m64, k.wcoef[wall][a], k.w[a]);
+        }
+    } else {
+        const float dh = __fadd_rn(sum.h, sum.m);
+        const float dl = __fadd_rn(__fsub_rn(sum.m, __fsub_rn(dh, sum.h)), sum.l);
+        bool sure = true;
+#pragma unroll
+        for (int l = 0; l < L::nout(); ++l) {
+            const KWall::Emit ce = kw.e[wall][l];
+            const float p = __fmul_rn(dh, ce.ch), e = __fmaf_rn(dh, ce.ch, -p);
+            const float t = __fmaf_rn(dh, ce.cl, __fmaf_rn(dl, ce.ch, e));
+            float v, r;
+            two_sum(ce.c0h, p, v, r);
+            const float z = __fadd_rn(r, __fadd_rn(ce.c0l, t));
+            // |error of v + z| < 2^-44 (|c0| + |p|): splits, products and sums
+            // of the low parts, each at most 2^-47 of them
+            const float eps = __fmul_rn(__fadd_rn(fabsf(ce.c0h), fabsf(p)), 0x1p-43f);
+            const float lo = __fadd_rn(v, __fsub_rn(z, eps)), hi = __fadd_rn(v, __fadd_rn(z, eps));
+            sure = sure && lo == hi;
+            out[l * stride] = lo;
+        }
+        if (!sure) wall_fill_exact<Q, PREC>(sum.h, sum.m, sum.l, k, kw, wall, out, stride);
+    }
 }
 
 // Specular partner of velocity a for fluid cell (x, j) next to a wall: the
 // mirrored velocity b = (e_x, -e_y) reaching the ghost node from which a leaves
 // came from the same row, 2 e_x columns back (periodic), in the collision's form.
+// (Out of line: rare, and inlined per velocity it would double the pull's code.)
 template <int PREC>
-__device__ __forceinline__ typename Store<PREC>::C
+__device__ __noinline__ typename Store<PREC>::C
 specular_source(const typename Store<PREC>::S *__restrict__ fin, const float *__restrict__ rin,
                 const KConsts<typename Store<PREC>::C> &k, int a, int ex, int x, int j) {
     const int b = k.mirror[a];

@@ -110,6 +110,20 @@ struct KConsts {
     unsigned long long wait_ns;
 };
 
+// Wall constants of the step kernels (wall 0 bottom, 1 top).  The velocities
+// leaving a wall: out_a[0][l], those with e_y > 0 in ascending order, out_a[1][l]
+// the opposite of out_a[0][l].  FP32 / BF16 formats: the l-th re-emission
+// M_in g^w_a / D_w (- w_a) as c0 + d c with d the sum of the incoming deviations,
+// c = g^w_a / D_w and c0 = (sum of the incoming terms' weights) c - w_a (BF16DEV:
+// d the whole sum, c0 = 0); c and c0 as pairs of floats.
+constexpr int kMaxWallOut = 16;   // 15 for D2Q37
+struct KWall {
+    struct Emit { float c0h, c0l, ch, cl; } e[2][kMaxWallOut];
+    double wsum[2];           // weights of the incoming terms (BF16DEV: 0)
+    int diffuse[2];           // accommodation 1
+    signed char out_a[2][kMaxWallOut];
+};
+
 // Constants of the FP64 one-warp-per-cell step by lane (k_step_cellwarp64.cuh):
 // lane 0 the rest velocity, lane p the pair (2p - 1, 2p), whose first member's
 // velocity is (ex, ey).
@@ -133,6 +147,7 @@ struct CellLanes {
 template <class C>
 void fill_consts(KConsts<C> &k, const LatticeHost &L, const lbm_params &p, int pitch);
 void fill_cell_lanes(CellLanes &c, const LatticeHost &L, const lbm_params &p);
+void fill_wall(KWall &kw, const LatticeHost &L, const lbm_params &p, const KConsts<float> &k);
 
 struct SolverImpl {
     LatticeHost L;
@@ -159,6 +174,7 @@ struct SolverImpl {
     double wall_in[2];
     KConsts<float> kf;
     KConsts<double> kd;
+    KWall kw;
     CellLanes lanes;
     int cell_cluster;         // many-step launch on one cluster: 0 not asked yet, 1 schedulable, -1 not
     int sm_count;
