@@ -176,33 +176,49 @@ int check_device_error(SolverImpl &s) {
     return LBM_OK;
 }
 
-int sum_rho(SolverImpl &s, double *out) {
-    const int nb = reduction_blocks((long long)s.p.Nx * s.p.Ny);
-    CU(dispatch_prec(s.p.precision, [&](auto P) { return Launch<decltype(P)::value>::mass_partials(s, s.red, nb); }));
-    CU(launch_final_sum(s.stream, s.red, nb, 1, s.red + 8 * 1024));
+int fetch_sum(SolverImpl &s, double *out) {
     CU(cudaMemcpyAsync(s.pinned, s.red + 8 * 1024, sizeof(double), cudaMemcpyDeviceToHost, s.stream));
     CU(cudaStreamSynchronize(s.stream));
     *out = s.pinned[0];
     return LBM_OK;
 }
 
-// The rounding counter of the current buffer holds the step count.
+int sum_rho(SolverImpl &s, double *out) {
+    const int nb = reduction_blocks((long long)s.p.Nx * s.p.Ny);
+    CU(dispatch_prec(s.p.precision, [&](auto P) { return Launch<decltype(P)::value>::mass_partials(s, s.red, nb); }));
+    CU(launch_final_sum(s.stream, s.red, nb, 1, s.red + 8 * 1024));
+    return fetch_sum(s, out);
+}
+
+// The rounding counter of the current buffer holds the step count (enqueued;
+// pinned[63] is free again once the stream has been waited for).
 int set_round_counter(SolverImpl &s) {
     s.pinned[63] = 0.0;
     unsigned v = (unsigned)s.steps;
     std::memcpy(&s.pinned[63], &v, sizeof v);
     CU(cudaMemcpyAsync(s.sr + s.cur, &s.pinned[63], sizeof(unsigned), cudaMemcpyHostToDevice, s.stream));
-    CU(cudaStreamSynchronize(s.stream));
     return LBM_OK;
 }
 
-int after_init(SolverImpl &s) {
+// A new state from device planes (rho NULL: lbm_solver_init's); synchronous.
+int init_state(SolverImpl &s, const double *rho, const double *ux, const double *uy,
+               const double *T) {
+    int nb = 0;
+    // the fifth staging plane is free: at most four hold the fields
+    double *partials = s.stage + 4 * (size_t)s.p.Nx * s.p.Ny;
+    CU(dispatch_prec(s.p.precision, [&](auto P) {
+        return Launch<decltype(P)::value>::init(s, rho, ux, uy, T, partials, &nb);
+    }));
     s.steps = 0;
-    if (int rc = set_round_counter(s)) return rc;
     s.last_res = -1;
-    int rc = sum_rho(s, &s.mass0);
-    if (rc) return rc;
-    // previous-check planes of the residual start from the initial fields
+    if (int rc = set_round_counter(s)) return rc;
+    // at most 2^31 / (17 x 16) blocks (the narrowest rows): red holds their groups
+    CU(launch_sum_many(s.stream, partials, nb, s.red, s.red + 8 * 1024));
+    return fetch_sum(s, &s.mass0);
+}
+
+// previous-check planes of the residual from the current state
+int fields_to_prev(SolverImpl &s) {
     const long long n = (long long)s.p.Nx * s.p.Ny;
     CU(dispatch_prec(s.p.precision, [&](auto P) {
         return Launch<decltype(P)::value>::macros(s, nullptr, s.prev, nullptr, s.prev + n);
@@ -341,8 +357,7 @@ int direct_variant_count(int precision) {
 }
 
 int dispatch_init_rest(SolverImpl &s) {
-    CU(dispatch_prec(s.p.precision, [&](auto P) { return Launch<decltype(P)::value>::init_rest(s); }));
-    return after_init(s);
+    return init_state(s, nullptr, nullptr, nullptr, nullptr);
 }
 
 int launch_step_variant(SolverImpl &s, int src, int dst, int kernel, int variant) {
@@ -585,9 +600,7 @@ int lbm_solver_destroy(lbm_solver *h) {
 int lbm_solver_init(lbm_solver *h) {
     API_BEGIN
     if (!h) { set_error("NULL solver"); return LBM_EINVAL; }
-    SolverImpl &s = h->s;
-    CU(dispatch_prec(s.p.precision, [&](auto P) { return Launch<decltype(P)::value>::init_rest(s); }));
-    return after_init(s);
+    return init_state(h->s, nullptr, nullptr, nullptr, nullptr);
     API_END
 }
 
@@ -604,10 +617,7 @@ int lbm_solver_init_fields(lbm_solver *h, const double *rho, const double *ux, c
             dst[i] = s.stage + i * n;
             CU(cudaMemcpyAsync(dst[i], src[i], n * sizeof(double), cudaMemcpyHostToDevice, s.stream));
         }
-    CU(dispatch_prec(s.p.precision, [&](auto P) {
-        return Launch<decltype(P)::value>::init_fields(s, dst[0], dst[1], dst[2], dst[3]);
-    }));
-    return after_init(s);
+    return init_state(s, dst[0], dst[1], dst[2], dst[3]);
     API_END
 }
 
@@ -730,8 +740,11 @@ int lbm_solver_set_f(lbm_solver *h, const double *f) {
         CU(cudaMemcpyAsync(s.stage, f + a * n, n * sizeof(double), cudaMemcpyHostToDevice, s.stream));
         CU(dispatch_prec(s.p.precision, [&](auto P) { return Launch<decltype(P)::value>::plane_from_f64(s, a, s.stage); }));
     }
-    CU(cudaStreamSynchronize(s.stream));
-    return after_init(s);
+    s.steps = 0;
+    s.last_res = -1;
+    if (int rc = set_round_counter(s)) return rc;
+    if (int rc = sum_rho(s, &s.mass0)) return rc;
+    return fields_to_prev(s);
     API_END
 }
 
@@ -860,10 +873,7 @@ int lbm_solver_set_state(lbm_solver *h, const void *buf, size_t bytes) {
     s.steps = hd.steps;
     s.mass0 = hd.mass0;
     if (int rc = set_round_counter(s)) return rc;
-    const long long n = (long long)s.p.Nx * s.p.Ny;
-    CU(dispatch_prec(s.p.precision, [&](auto P) {
-        return Launch<decltype(P)::value>::macros(s, nullptr, s.prev, nullptr, s.prev + n);
-    }));
+    if (int rc = fields_to_prev(s)) return rc;
     CU(cudaStreamSynchronize(s.stream));
     return LBM_OK;
     API_END

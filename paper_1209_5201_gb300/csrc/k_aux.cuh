@@ -25,7 +25,7 @@ __device__ __forceinline__ double splitmix_u01(uint64_t seed, uint64_t k) {
 template <int Q, class C, bool SHIFT>
 __device__ __forceinline__ void equilibrium_all(C rho, C drho, C ux, C uy, C T,
                                                 const KConsts<C> &k, C (&o)[Q]) {
-    // A collision with omega = 1 from f = 0 leaves exactly rho g^eq.
+    // the equilibrium terms of a collision with omega = 1
     Collision<Q, C, SHIFT> col;
     const C u2 = ux * ux + uy * uy;
     col.set_omega(C(1));
@@ -33,64 +33,126 @@ __device__ __forceinline__ void equilibrium_all(C rho, C drho, C ux, C uy, C T,
     col.sy = k.r * uy;
     col.rho = rho;
     col.set_coefficients(u2, T - C(1), rho, drho / rho, k);
-    o[0] = col.rest(C(0));
+    o[0] = col.cw[0] * col.A0[0];
     PairLoop<1, Q>::run([&](auto ic) {
         constexpr int A = decltype(ic)::value;
-        col.template pair<A>(C(0), C(0), o[A], o[A + 1]);
+        C P, R;
+        col.template eq_pair<A>(P, R);
+        o[A] = P + R;
+        o[A + 1] = P - R;
     });
 }
 
-template <int Q, int PREC>
-__device__ __forceinline__ void store_cell(typename Store<PREC>::S *f, float *rplane,
-                                           const KConsts<typename Store<PREC>::C> &k, int x,
-                                           int j, const typename Store<PREC>::C (&o)[Q],
-                                           typename Store<PREC>::C rho) {
-    using S = typename Store<PREC>::S;
-    using C = typename Store<PREC>::C;
+// Eq. (3) fields of a cell from its stored values v (deviations where the
+// format stores them; BF16DEV: its density rc): rho, u_x, u_y and the kinetic
+// temperature sum f |c - u|^2 / (2 rho), in the storage's compute type.
+template <int Q, int PREC, class C>
+__device__ __forceinline__ void cell_fields(const C (&sv)[Q], C rc, const KConsts<C> &k,
+                                            double (&o)[4]) {
+    using L = Lat<Q>;
+    C s0 = 0, sx = 0, sy = 0, se = 0;
+    if constexpr (PREC == LBM_FP64) {
+        // FP64 instructions are the cost: sums and differences of opposite
+        // pairs, and one reciprocal: about 115 of them instead of 175
+        s0 = sv[0];
+        PairLoop<1, Q>::run([&](auto ic) {
+            constexpr int A = decltype(ic)::value;
+            const C s = sv[A] + sv[A + 1], d = sv[A] - sv[A + 1];
+            s0 += s;
+            if constexpr (L::ex(A) != 0) sx += C(L::ex(A)) * d;
+            if constexpr (L::ey(A) != 0) sy += C(L::ey(A)) * d;
+            se += C(L::e2(A)) * s;
+        });
+    } else {
 #pragma unroll
-    for (int a = 0; a < Q; ++a) {
-        C v = o[a];
-        if constexpr (Store<PREC>::dev) v -= k.w[a] * rho;
-        store_pop<S>(f, k, a, j, x, from_c<S>(v));
+        for (int a = 0; a < Q; ++a) {
+            C v = sv[a];
+            if constexpr (Store<PREC>::dev) v += k.w[a] * rc;
+            s0 += v;
+            sx += C(L::ex(a)) * v;
+            sy += C(L::ey(a)) * v;
+            se += C(L::e2(a)) * v;
+        }
     }
-    if constexpr (Store<PREC>::dev) store_rho(rplane, k, j, x, (float)rho);
+    // shifted storage: the sums are of deviations; sum w = 1, sum e w = 0
+    const C rh = Store<PREC>::shifted ? C(1) + s0 : s0;
+    // rho D T = sum f |c - u|^2 = r^2 sum e^2 f - rho u^2
+    if constexpr (PREC == LBM_FP64) {
+        const C inv = __drcp_rn(rh), u = k.r * sx * inv, v = k.r * sy * inv;
+        o[0] = rh;
+        o[1] = u;
+        o[2] = v;
+        o[3] = 0.5 * (k.r2 * se * inv - (u * u + v * v));
+    } else {
+        const C u = k.r * sx / rh, v = k.r * sy / rh;
+        if constexpr (Store<PREC>::shifted) se += k.e2w;
+        const C e = k.r2 * se - rh * (u * u + v * v);
+        o[0] = (double)rh;
+        o[1] = (double)u;
+        o[2] = (double)v;
+        o[3] = (double)(e / (C(2) * rh));
+    }
 }
 
-// f~* = rho0 (1 + amp (2U - 1)) g^eq(0, 1) = rho w_a.
-template <int Q, int PREC>
-__global__ void k_init_rest(typename Store<PREC>::S *f, float *rplane,
-                            const __grid_constant__ KConsts<typename Store<PREC>::C> k,
-                            double rho0, double amp, uint64_t seed) {
-    using C = typename Store<PREC>::C;
-    const long long n = (long long)k.Nx * k.Ny;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
-         c += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(c / k.Nx), x = (int)(c % k.Nx);
-        double rho = rho0;
-        if (amp != 0.0) rho = rho0 * (1.0 + amp * (2.0 * splitmix_u01(seed, (uint64_t)c) - 1.0));
-        C o[Q];
-        equilibrium_all<Q, C, Store<PREC>::shifted>((C)rho, (C)(rho - 1.0), C(0), C(0), C(1), k, o);
-        store_cell<Q, PREC>(f, rplane, k, x, j, o, (C)rho);
+// sum of rho over a cell's stored values.  FP32 / BF16: the stored deviations
+// are summed in FP32 (they are small, so its rounding is far below FP32
+// resolution of the cell's mass) and the rest is added in FP64; FP64 storage
+// sums in FP64.  wsum: FP64 sum of the weights (BF16DEV).
+template <int Q, int PREC, class C>
+__device__ __forceinline__ double cell_mass(const C (&sv)[Q], double wsum, float rc) {
+    C sd = 0;
+#pragma unroll
+    for (int a = 0; a < Q; ++a) sd += sv[a];
+    double s = (double)sd;
+    if constexpr (Store<PREC>::shifted) s += 1.0;            // sum of the weights
+    if constexpr (Store<PREC>::dev) s += wsum * (double)rc;
+    return s;
+}
+
+// Block-level FP64 sum of NV values per thread (warp shuffle, then shared).
+template <int NV>
+__device__ __forceinline__ void block_sum(double (&v)[NV], double *out) {
+    __shared__ double sh[32][NV];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+        for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_down_sync(0xffffffffu, v[i], o);
+    if (lane == 0)
+        for (int i = 0; i < NV; ++i) sh[wid][i] = v[i];
+    __syncthreads();
+    if (wid == 0) {
+        const int nw = (blockDim.x + 31) >> 5;
+        for (int i = 0; i < NV; ++i) {
+            double s = lane < nw ? sh[lane][i] : 0.0;
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+            if (lane == 0) out[i] = s;
+        }
     }
 }
 
-// f~* = rho g^eq(u, T) from FP64 device planes [Ny][Nx] (NULL: u = 0, T = 1).
-template <int Q, int PREC>
-__global__ void k_init_fields(typename Store<PREC>::S *f, float *rplane,
-                              const __grid_constant__ KConsts<typename Store<PREC>::C> k,
-                              const double *rho, const double *ux, const double *uy,
-                              const double *T) {
-    using C = typename Store<PREC>::C;
-    const long long n = (long long)k.Nx * k.Ny;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
-         c += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(c / k.Nx), x = (int)(c % k.Nx);
-        C o[Q];
-        equilibrium_all<Q, C, Store<PREC>::shifted>((C)rho[c], (C)(rho[c] - 1.0),
-                                                    ux ? (C)ux[c] : C(0), uy ? (C)uy[c] : C(0),
-                                                    T ? (C)T[c] : C(1), k, o);
-        store_cell<Q, PREC>(f, rplane, k, x, j, o, (C)rho[c]);
+// Block sum of one FP32 value per thread to FP64 precision by error-free
+// additions of float pairs (an FP64 add, or a conversion, takes a warp 64
+// cycles); the result in thread 0.
+__device__ __forceinline__ double block_sum_f32(float v) {
+    __shared__ float sh[32][2];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    float h = v, l = 0.0f;
+    auto merge = [&](float h2, float l2) {
+        float e;
+        two_sum(h, h2, h, e);
+        l = __fadd_rn(__fadd_rn(l, l2), e);
+    };
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float h2 = __shfl_down_sync(0xffffffffu, h, o), l2 = __shfl_down_sync(0xffffffffu, l, o);
+        merge(h2, l2);
     }
+    __syncthreads();                         // sh may still be read by a call before
+    if (lane == 0) sh[wid][0] = h, sh[wid][1] = l;
+    __syncthreads();
+    if (threadIdx.x != 0) return 0.0;
+    for (int i = 1; i < (int)(blockDim.x + 31) / 32; ++i) merge(sh[i][0], sh[i][1]);
+    return (double)h + (double)l;
 }
 
 // Velocity plane a of the stored state -> FP64 logical plane [Ny][Nx].
@@ -138,39 +200,22 @@ template <int Q, int PREC>
 __global__ void k_macros(const typename Store<PREC>::S *f, const float *rplane,
                          const __grid_constant__ KConsts<typename Store<PREC>::C> k,
                          double *rho, double *ux, double *uy, double *T, int acc) {
-    using L = Lat<Q>;
     using C = typename Store<PREC>::C;
     const long long n = (long long)k.Nx * k.Ny;
-    const C r = k.r;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
          c += (long long)gridDim.x * blockDim.x) {
         const int j = (int)(c / k.Nx), x = (int)(c % k.Nx);
         const long long ro = col_index(k, j, x);
-        const long long rr = rho_index(k, j, x);
-        C fv[Q];
-        C s0 = 0, sx = 0, sy = 0, se = 0;
+        C v[Q], rc = 0;
 #pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            C v = to_c(f[ro + (long long)a * k.pitch]);
-            if constexpr (Store<PREC>::dev) v += k.w[a] * rplane[rr];
-            fv[a] = v;
-            s0 += v;
-            sx += C(L::ex(a)) * v;
-            sy += C(L::ey(a)) * v;
-            se += C(L::e2(a)) * v;
-        }
-        // shifted storage: the sums are of deviations; sum w = 1, sum e w = 0
-        const C rh = Store<PREC>::shifted ? C(1) + s0 : s0;
-        const C u = r * sx / rh, v = r * sy / rh;
-        if constexpr (Store<PREC>::shifted) se += k.e2w;
-        // rho D T = sum f |c - u|^2 = r^2 sum e^2 f - rho u^2
-        const C e = k.r2 * se - rh * (u * u + v * v);
-        const double o[4] = {(double)rh, (double)u, (double)v, (double)(e / (C(2) * rh))};
+        for (int a = 0; a < Q; ++a) v[a] = to_c(f[ro + (long long)a * k.pitch]);
+        if constexpr (Store<PREC>::dev) rc = rplane[rho_index(k, j, x)];
+        double o[4];
+        cell_fields<Q, PREC, C>(v, rc, k, o);
         double *out[4] = {rho, ux, uy, T};
 #pragma unroll
         for (int i = 0; i < 4; ++i)
             if (out[i]) out[i][c] = acc ? out[i][c] + o[i] : o[i];
-        (void)fv;
     }
 }
 
@@ -203,60 +248,27 @@ __global__ void k_wall_mass(const typename Store<PREC>::S *f, const float *rplan
     }
 }
 
-// Block-level FP64 sum of NV values per thread (warp shuffle, then shared).
-template <int NV>
-__device__ __forceinline__ void block_sum(double (&v)[NV], double *out) {
-    __shared__ double sh[32][NV];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < NV; ++i)
-        for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_down_sync(0xffffffffu, v[i], o);
-    if (lane == 0)
-        for (int i = 0; i < NV; ++i) sh[wid][i] = v[i];
-    __syncthreads();
-    if (wid == 0) {
-        const int nw = (blockDim.x + 31) >> 5;
-        for (int i = 0; i < NV; ++i) {
-            double s = lane < nw ? sh[lane][i] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-            if (lane == 0) out[i] = s;
-        }
-    }
-}
-
-// Sum of rho over all cells: per-block partials (fixed grid, fixed order).
+// Sum of rho over all cells: per-block partials (fixed grid, fixed order).  A
+// block takes whole rows, several at a time where they are narrower than the
+// block (one division per thread, none per cell).
 template <int Q, int PREC>
 __global__ void k_mass_partials(const typename Store<PREC>::S *f, const float *rplane,
                                 const __grid_constant__ KConsts<typename Store<PREC>::C> k,
-                                double *partials) {
-    // rows j = blockIdx.x, + gridDim.x, ...; the block's threads stride over x
-    // (no division per cell).  FP32 / BF16DEV storage: a cell's sum of stored
-    // deviations is formed in FP32 (they are small, so its rounding is far
-    // below FP32 resolution of the cell's mass) and added to an FP64 total;
-    // FP64 storage sums in FP64.
+                                double wsum, double *partials) {
+    using C = typename Store<PREC>::C;
     double acc[1] = {0.0};
-    double wsum = 0.0;
-    if constexpr (Store<PREC>::dev) {
-#pragma unroll
-        for (int a = 0; a < Q; ++a) wsum += (double)k.w[a];
-    }
-    for (int j = blockIdx.x; j < k.Ny; j += gridDim.x) {
-        for (int x = threadIdx.x; x < k.Nx; x += blockDim.x) {
+    const int rows = k.Nx < (int)blockDim.x ? blockDim.x / k.Nx : 1;
+    const int tr = rows > 1 ? threadIdx.x / k.Nx : 0, tx = threadIdx.x - tr * k.Nx;
+    const int x0 = rows > 1 ? (tr < rows ? tx : k.Nx) : threadIdx.x;
+    for (int j = blockIdx.x * rows + tr; j < k.Ny; j += gridDim.x * rows) {
+        for (int x = x0; x < k.Nx; x += blockDim.x) {
             const typename Store<PREC>::S *cell = f + col_index(k, j, x);
-            if constexpr (PREC == LBM_FP64) {
-                double s = 0.0;
+            C v[Q];
 #pragma unroll
-                for (int a = 0; a < Q; ++a) s += cell[(long long)a * k.pitch];
-                acc[0] += s;
-            } else {
-                float sd = 0.0f;
-#pragma unroll
-                for (int a = 0; a < Q; ++a) sd += to_c(cell[(long long)a * k.pitch]);
-                double s = (double)sd;
-                if constexpr (Store<PREC>::shifted) s += 1.0;    // sum of the weights
-                if constexpr (Store<PREC>::dev) s += wsum * (double)rplane[rho_index(k, j, x)];
-                acc[0] += s;
-            }
+            for (int a = 0; a < Q; ++a) v[a] = to_c(cell[(long long)a * k.pitch]);
+            float rc = 0.0f;
+            if constexpr (Store<PREC>::dev) rc = rplane[rho_index(k, j, x)];
+            acc[0] += cell_mass<Q, PREC, C>(v, wsum, rc);
         }
     }
     block_sum<1>(acc, partials + blockIdx.x);

@@ -69,6 +69,29 @@ int launch_rho_plane(cudaStream_t st, float *rplane, const double *acc, const KC
     return (int)cudaGetLastError();
 }
 
+// Partials of a group of 1024 (one block each): out[block].
+__global__ void k_group_sum(const double *partials, int n, double *out) {
+    double v[1] = {0.0};
+    const int i0 = blockIdx.x * 1024 + threadIdx.x;
+#pragma unroll
+    for (int i = 0; i < 1024 / kAuxThreads; ++i)
+        if (i0 + i * kAuxThreads < n) v[0] += partials[i0 + i * kAuxThreads];
+    block_sum<1>(v, out + blockIdx.x);
+}
+
+// One value per block of a large grid: first by groups of 1024 (65 536
+// partials: 33 us in one block), groups + n doubles behind `partials`.
+int launch_sum_many(cudaStream_t st, double *partials, int n, double *groups, double *out) {
+    const double *in = partials;
+    for (; n > 4096; n = (n + 1023) / 1024) {
+        double *to = in == groups ? partials : groups;
+        k_group_sum<<<(n + 1023) / 1024, kAuxThreads, 0, st>>>(in, n, to);
+        in = to;
+    }
+    k_final_sum<<<1, kAuxThreads, 0, st>>>(in, n, 1, out);
+    return (int)cudaGetLastError();
+}
+
 int launch_final_sum(cudaStream_t st, const double *partials, int nblocks, int nv, double *out) {
     k_final_sum<<<1, kAuxThreads, 0, st>>>(partials, nblocks, nv, out);
     return (int)cudaGetLastError();

@@ -15,9 +15,10 @@ struct Launch {
     // n steps in one launch; cudaErrorNotSupported: use step_cellwarp
     static int steps_cellwarp(SolverImpl &s, int src, int n);
     static int staged_variants();
-    static int init_rest(SolverImpl &s);
-    static int init_fields(SolverImpl &s, const double *rho, const double *ux,
-                           const double *uy, const double *T);
+    // the state rho g^eq(u, T) (rho NULL: lbm_solver_init's), the fields of the
+    // first residual check and *nblocks (<= Nx Ny) block partials of the mass
+    static int init(SolverImpl &s, const double *rho, const double *ux, const double *uy,
+                    const double *T, double *partials, int *nblocks);
     static int plane_to_f64(SolverImpl &s, int a, double *out);
     static int plane_from_f64(SolverImpl &s, int a, const double *in);
     // Eq. (3) fields into FP64 device planes; acc = 1 adds them instead
@@ -33,6 +34,8 @@ struct Launch {
 int launch_accumulate(cudaStream_t st, double *acc, const double *in, long long n, int first);
 int launch_rho_plane(cudaStream_t st, float *rplane, const double *acc, const KConsts<float> &k);
 int launch_final_sum(cudaStream_t st, const double *partials, int nblocks, int nv, double *out);
+// sum of n partials (overwritten) in a fixed order; groups: room for n / 1024 + 1
+int launch_sum_many(cudaStream_t st, double *partials, int n, double *groups, double *out);
 int launch_residual_partials(cudaStream_t st, const double *ux, const double *T, double *uxp,
                              double *Tp, long long n, double Tref, double *partials,
                              int nblocks);

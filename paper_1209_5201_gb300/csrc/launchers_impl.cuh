@@ -3,6 +3,7 @@
 
 #include "k_aux.cuh"
 #include "k_fluxes.cuh"
+#include "k_init.cuh"
 #include "k_step_cellwarp.cuh"
 #include "k_step_cellwarp64.cuh"
 #include "k_step_direct.cuh"
@@ -25,6 +26,13 @@ template <> struct Consts<LBM_BF16DEV> {
 template <> struct Consts<LBM_BF16SHIFT> {
     static const KConsts<float> &get(const SolverImpl &s) { return s.kf; }
 };
+
+template <class C>
+double weight_sum(const KConsts<C> &k) {
+    double s = 0.0;
+    for (int a = 0; a < k.Q; ++a) s += (double)k.w[a];
+    return s;
+}
 
 inline int aux_blocks(long long n) {
     long long b = (n + kAuxThreads - 1) / kAuxThreads;
@@ -300,24 +308,16 @@ int Launch<PREC>::step_staged(SolverImpl &s, int src, int dst, int variant) {
 }
 
 template <int PREC>
-int Launch<PREC>::init_rest(SolverImpl &s) {
+int Launch<PREC>::init(SolverImpl &s, const double *rho, const double *ux, const double *uy,
+                       const double *T, double *partials, int *nblocks) {
     using S = typename Store<PREC>::S;
     const auto &k = Consts<PREC>::get(s);
-    const long long n = (long long)s.p.Nx * s.p.Ny;
-    LBM_DISPATCH_Q(s.L.Q, (k_init_rest<QQ, PREC><<<aux_blocks(n), kAuxThreads, 0, s.stream>>>(
-                               (S *)s.f[s.cur], s.rho[s.cur], k, s.p.rho0, s.p.noise_amp,
-                               s.p.seed)));
-    return (int)cudaGetLastError();
-}
-
-template <int PREC>
-int Launch<PREC>::init_fields(SolverImpl &s, const double *rho, const double *ux,
-                              const double *uy, const double *T) {
-    using S = typename Store<PREC>::S;
-    const auto &k = Consts<PREC>::get(s);
-    const long long n = (long long)s.p.Nx * s.p.Ny;
-    LBM_DISPATCH_Q(s.L.Q, (k_init_fields<QQ, PREC><<<aux_blocks(n), kAuxThreads, 0, s.stream>>>(
-                               (S *)s.f[s.cur], s.rho[s.cur], k, rho, ux, uy, T)));
+    *nblocks = (int)init_blocks(k);
+    double *prev_u = s.prev, *prev_T = s.prev + (long long)s.p.Nx * s.p.Ny;
+    LBM_DISPATCH_Q(s.L.Q, (k_init<QQ, PREC><<<*nblocks, kInitThreads, 0, s.stream>>>(
+                               (S *)s.f[s.cur], s.rho[s.cur], k, rho, ux, uy, T, s.p.rho0,
+                               s.p.noise_amp, s.p.seed, prev_u, prev_T, weight_sum(k),
+                               partials)));
     return (int)cudaGetLastError();
 }
 
@@ -379,7 +379,7 @@ int Launch<PREC>::mass_partials(SolverImpl &s, double *partials, int nblocks) {
     using S = typename Store<PREC>::S;
     const auto &k = Consts<PREC>::get(s);
     LBM_DISPATCH_Q(s.L.Q, (k_mass_partials<QQ, PREC><<<nblocks, kAuxThreads, 0, s.stream>>>(
-                               (const S *)s.f[s.cur], s.rho[s.cur], k, partials)));
+                               (const S *)s.f[s.cur], s.rho[s.cur], k, weight_sum(k), partials)));
     return (int)cudaGetLastError();
 }
 

@@ -7,9 +7,8 @@ template int Launch<LBM_BF16DEV>::step_staged(SolverImpl &, int, int, int);
 template int Launch<LBM_BF16DEV>::step_cellwarp(SolverImpl &, int, int);
 template int Launch<LBM_BF16DEV>::steps_cellwarp(SolverImpl &, int, int);
 template int Launch<LBM_BF16DEV>::staged_variants();
-template int Launch<LBM_BF16DEV>::init_rest(SolverImpl &);
-template int Launch<LBM_BF16DEV>::init_fields(SolverImpl &, const double *, const double *,
-                                      const double *, const double *);
+template int Launch<LBM_BF16DEV>::init(SolverImpl &, const double *, const double *, const double *,
+                                     const double *, double *, int *);
 template int Launch<LBM_BF16DEV>::plane_to_f64(SolverImpl &, int, double *);
 template int Launch<LBM_BF16DEV>::plane_from_f64(SolverImpl &, int, const double *);
 template int Launch<LBM_BF16DEV>::macros(SolverImpl &, double *, double *, double *, double *, int);

@@ -7,9 +7,8 @@ template int Launch<LBM_BF16SHIFT>::step_staged(SolverImpl &, int, int, int);
 template int Launch<LBM_BF16SHIFT>::step_cellwarp(SolverImpl &, int, int);
 template int Launch<LBM_BF16SHIFT>::steps_cellwarp(SolverImpl &, int, int);
 template int Launch<LBM_BF16SHIFT>::staged_variants();
-template int Launch<LBM_BF16SHIFT>::init_rest(SolverImpl &);
-template int Launch<LBM_BF16SHIFT>::init_fields(SolverImpl &, const double *, const double *,
-                                      const double *, const double *);
+template int Launch<LBM_BF16SHIFT>::init(SolverImpl &, const double *, const double *, const double *,
+                                     const double *, double *, int *);
 template int Launch<LBM_BF16SHIFT>::plane_to_f64(SolverImpl &, int, double *);
 template int Launch<LBM_BF16SHIFT>::plane_from_f64(SolverImpl &, int, const double *);
 template int Launch<LBM_BF16SHIFT>::macros(SolverImpl &, double *, double *, double *, double *, int);

@@ -7,9 +7,8 @@ template int Launch<LBM_FP32>::step_staged(SolverImpl &, int, int, int);
 template int Launch<LBM_FP32>::step_cellwarp(SolverImpl &, int, int);
 template int Launch<LBM_FP32>::steps_cellwarp(SolverImpl &, int, int);
 template int Launch<LBM_FP32>::staged_variants();
-template int Launch<LBM_FP32>::init_rest(SolverImpl &);
-template int Launch<LBM_FP32>::init_fields(SolverImpl &, const double *, const double *,
-                                      const double *, const double *);
+template int Launch<LBM_FP32>::init(SolverImpl &, const double *, const double *, const double *,
+                                     const double *, double *, int *);
 template int Launch<LBM_FP32>::plane_to_f64(SolverImpl &, int, double *);
 template int Launch<LBM_FP32>::plane_from_f64(SolverImpl &, int, const double *);
 template int Launch<LBM_FP32>::macros(SolverImpl &, double *, double *, double *, double *, int);
