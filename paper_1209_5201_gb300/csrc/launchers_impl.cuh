@@ -358,8 +358,20 @@ int Launch<PREC>::fluxes(SolverImpl &s, double *sxx, double *sxy, double *syy, d
     using S = typename Store<PREC>::S;
     const auto &k = Consts<PREC>::get(s);
     dim3 grid((s.p.Nx + kFluxThreads - 1) / kFluxThreads, s.p.Ny);
+    LatticeMoments lm = {};
+    lm.h_tau = 0.5 / s.kd.tau_lat;
+    lm.h_rho = 0.5 / s.kd.K;
+    for (int a = 0; a < s.L.Q; ++a) {
+        const double w = s.L.w[a], x2 = s.L.ex[a] * s.L.ex[a], y2 = s.L.ey[a] * s.L.ey[a];
+        lm.m00 += w;
+        lm.m20 += w * x2;
+        lm.m40 += w * x2 * x2;
+        lm.m22 += w * x2 * y2;
+        lm.m60 += w * x2 * x2 * x2;
+        lm.m42 += w * x2 * x2 * y2;
+    }
     LBM_DISPATCH_Q(s.L.Q, (k_fluxes<QQ, PREC><<<grid, kFluxThreads, 0, s.stream>>>(
-                               (const S *)s.f[s.cur], s.rho[s.cur], k, s.kw, s.kd, sxx, sxy, syy, qx,
+                               (const S *)s.f[s.cur], s.rho[s.cur], k, s.kw, s.kd, lm, sxx, sxy, syy, qx,
                                qy)));
     return (int)cudaGetLastError();
 }
