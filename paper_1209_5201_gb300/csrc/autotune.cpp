@@ -1,7 +1,8 @@
 // Tile / block-shape autotuner of the step kernel.
 //
 // Candidates: every variant of the one-pass direct kernel and of the TMA-staged one compiled
-// for the solver's precision, and the one-warp-per-cell kernel on small grids.  Each runs `trial` steps after two warm-up
+// for the solver's precision, which round alike; in FP64 also the one-warp-per-cell kernel.
+// FP32 and BF16 grids take the latter by size alone (cellwarp_cells).  Each runs `trial` steps after two warm-up
 // steps, timed with CUDA events on the solver's stream; the fastest wins.
 // Results are cached per (lattice, precision, order, Nx class, Ny class) for
 // the life of the process and, when LBM_AUTOTUNE_CACHE names a file, across
@@ -89,15 +90,37 @@ int time_candidate(SolverImpl &s, int kernel, int variant, int trial, double *ms
     return rc;
 }
 
+// Cells up to which a tuned FP32 or BF16 grid takes the one-warp-per-cell
+// kernel.  That kernel sums the moments in another order than the others, so
+// the choice shows in the results (at FP32 round-off; in BF16 through the
+// rounding of what is stored) and is made by size, not by a timing that differs
+// from run to run.  The line lies where it was the faster one (us per step on
+// square grids, one warp per cell / one thread per cell): FP32 D2Q37 16 / 16.6 at
+// 6000 cells, 17 / 16.7 at 7000; D2Q25 12.3 / 12.5 at 5000; D2Q17 never; BF16DEV
+// D2Q37 26 / 27 at 12 000, D2Q25 18.4 / 18.7 at 10 000; BF16SHIFT D2Q37 22 / 25 at
+// 10 000, D2Q25 15.8 / 17.3 at 8000.  (The one-thread kernels' wall rows have
+// become three times faster since; moving the line would change results.)
+long long cellwarp_cells(int Q, int precision) {
+    const int i = Q == 37 ? 0 : Q == 25 ? 1 : 2;
+    constexpr long long fp32[3] = {6500, 4800, 0}, dev[3] = {13000, 9700, 3700},
+                        shift[3] = {11000, 9000, 2700};
+    return precision == LBM_FP32 ? fp32[i] : precision == LBM_BF16DEV ? dev[i] : shift[i];
+}
+
 }  // namespace
 
 int autotune_solver(SolverImpl &s, int trial) {
     const std::string key = class_key(s);
+    const long long cells = (long long)s.p.Nx * s.p.Ny;
+    const bool by_size = s.p.precision != LBM_FP64;
+    const bool small = by_size && cells <= cellwarp_cells(s.L.Q, s.p.precision);
     {
+        // (a size class may straddle the line: the other kernel's entry is not its)
         std::lock_guard<std::mutex> lk(g_mu);
         load_file_cache();
         auto it = g_cache.find(key);
-        if (it != g_cache.end()) {
+        if (it != g_cache.end() &&
+            (!by_size || small == (it->second.kernel == LBM_KERNEL_CELLWARP))) {
             s.p.kernel = it->second.kernel;
             s.variant = it->second.variant;
             s.tuned_ms = it->second.ms;
@@ -109,19 +132,19 @@ int autotune_solver(SolverImpl &s, int trial) {
     if (rc) return rc;
     Choice best{LBM_KERNEL_DIRECT, 0, 1e30};
     double ms = 0;
-    const int nd = direct_variant_count(s.p.precision);
+    const int nd = small ? 0 : direct_variant_count(s.p.precision);
     for (int v = 0; v < nd; ++v) {
         if ((rc = time_candidate(s, LBM_KERNEL_DIRECT, v, trial, &ms))) return rc;
         if (ms < best.ms) best = Choice{LBM_KERNEL_DIRECT, v, ms};
     }
     // the staged kernel: grids stored as one x-tile only
-    const int nv = s.nt == 1 ? staged_variant_count(s.p.precision) : 0;
+    const int nv = s.nt == 1 && !small ? staged_variant_count(s.p.precision) : 0;
     for (int v = 0; v < nv; ++v) {
         if ((rc = time_candidate(s, LBM_KERNEL_STAGED, v, trial, &ms))) return rc;
         if (ms < best.ms) best = Choice{LBM_KERNEL_STAGED, v, ms};
     }
-    // one warp per cell: only a candidate for small grids (32 threads a cell)
-    if ((long long)s.p.Nx * s.p.Ny <= 16 * kCellwarpAutoCells) {
+    // one warp per cell: FP64, where it is timed on small grids (32 threads a cell)
+    if (by_size ? small : cells <= 16 * kCellwarpAutoCells) {
         if ((rc = time_candidate(s, LBM_KERNEL_CELLWARP, 0, trial, &ms))) return rc;
         if (ms < best.ms) best = Choice{LBM_KERNEL_CELLWARP, 0, ms};
     }
