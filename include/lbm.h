@@ -259,7 +259,8 @@ int lbm_solver_stats(lbm_solver *s, lbm_stats *st);
 
 /* Step-kernel selection.  LBM_KERNEL_DIRECT: one thread per cell, populations
  * pulled straight from global memory; its variants differ in block width,
- * register cap, rows per block and store cache policy.  LBM_KERNEL_STAGED: persistent tile
+ * register cap (variant 0: by format and lattice), rows per block and store
+ * cache policy.  LBM_KERNEL_STAGED: persistent tile
  * kernel whose producer warp stages each velocity's shifted source window
  * (tile plus the +-3-cell halo, rounded to 16 bytes in x) into shared memory
  * with TMA; `variant` picks one of the compiled tile shapes, 0 <= variant <
@@ -293,7 +294,8 @@ int lbm_solver_variant_count(lbm_solver *s, int32_t kernel, int32_t *n);
 int lbm_solver_kernel_info(lbm_solver *s, int32_t *kernel, int32_t *variant,
                            int32_t *nvariants);
 /* Autotuner: time trial_steps steps of every direct and every staged
- * variant on this solver's grid (CUDA events on the solver's stream), keep
+ * variant (FP64: and of the one-warp-per-cell kernel; FP32 and BF16 grids of a
+ * few thousand cells take that one by size) on this solver's grid (CUDA events on the solver's stream), keep
  * the fastest, and cache the choice per (lattice, precision, order, Nx and Ny
  * rounded up to powers of two) for the process, and in the file named by the
  * environment variable LBM_AUTOTUNE_CACHE when set.  Overwrites the state:

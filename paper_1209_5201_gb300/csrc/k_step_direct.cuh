@@ -159,7 +159,7 @@ __device__ __forceinline__ void store_cell(const typename Store<PREC>::S (&v)[Q]
 // tile of w columns — and store the result: its own slots (dst: its element
 // of velocity 0; rdst: its density, BF16DEV) and, for the kPadL columns at
 // either end of the tile, the halo copies.
-template <int Q, int PREC, bool CS, int PC>
+template <int Q, int PREC, bool CS, int PC, bool ISO2>
 __device__ __forceinline__ void collide_store(const typename Store<PREC>::C (&f)[Q],
                                               typename Store<PREC>::S *__restrict__ fout,
                                               float *__restrict__ rout,
@@ -170,7 +170,7 @@ __device__ __forceinline__ void collide_store(const typename Store<PREC>::C (&f)
     using S = typename Store<PREC>::S;
     using C = typename Store<PREC>::C;
     const uint32_t hcell = Store<PREC>::sr ? sr_cell(seed, (uint32_t)j * (uint32_t)k.Nx + (uint32_t)x) : 0u;
-    Collision<Q, C, Store<PREC>::shifted> col;
+    Collision<Q, C, Store<PREC>::shifted, ISO2> col;
     col.setup(f, k);
     C o[Q];
     o[0] = col.rest(f[0]);
@@ -209,9 +209,10 @@ __device__ __forceinline__ void collide_store(const typename Store<PREC>::C (&f)
 // BX threads per block (one row segment of a tile); MINB blocks per SM
 // requested from the register allocator; CS: streaming stores; RS rows per
 // block, walked in order (rows [RS blockIdx.y, RS blockIdx.y + RS)); PC: the
-// tile pitch as a compile-time constant (0: the solver's).  Grid: blockIdx.x
+// tile pitch as a compile-time constant (0: the solver's); ISO2: the
+// second-order isothermal equilibrium compiled in.  Grid: blockIdx.x
 // = tile * ceil(tw / BX) + block of the tile.
-template <int Q, int PREC, int BX, int MINB, bool CS, int RS, int PC>
+template <int Q, int PREC, int BX, int MINB, bool CS, int RS, int PC, bool ISO2>
 __global__ void __launch_bounds__(BX, MINB)
 k_step_direct(const typename Store<PREC>::S *__restrict__ fin,
               typename Store<PREC>::S *__restrict__ fout, const float *__restrict__ rin,
@@ -263,7 +264,7 @@ k_step_direct(const typename Store<PREC>::S *__restrict__ fin,
                                         s_fill[RS > 1 && j >= L::N ? 1 : 0], f);
         else
             pull<Q, PREC, BX, false, PC>(fin, rin, fin + cell, rsrc, k, kw, x, j, s_fill[0], f);
-        collide_store<Q, PREC, CS, PC>(f, fout, rout, fout + cell, rdst, k, t, xl, w, x, j, seed);
+        collide_store<Q, PREC, CS, PC, ISO2>(f, fout, rout, fout + cell, rdst, k, t, xl, w, x, j, seed);
     }
 }
 

@@ -49,12 +49,28 @@ inline int aux_blocks(long long n) {
     }
 
 // ---- direct kernel variants {BX, MINB, CS, RS} ----------------------------------
-// RS: rows per block
+// RS: rows per block.  MINB < 0: the format's own choice (default_blocks).
 struct DirectVariants {
     static constexpr int n = 8;
-    static constexpr int v[n][4] = {{128, 0, 0, 1}, {128, 7, 0, 1}, {128, 6, 0, 1}, {256, 0, 0, 1},
+    static constexpr int v[n][4] = {{128, -1, 0, 1}, {128, 7, 0, 1}, {128, 6, 0, 1}, {256, 0, 0, 1},
                                     {128, 0, 1, 1}, {192, 0, 0, 1}, {128, 0, 0, 2}, {128, 5, 0, 1}};
 };
+// Blocks per SM that variant 0 asks the register allocator for, by what
+// measured fastest untuned, us per step on 4096 x 2048 / 2050 x 1023 /
+// 1000 x 500 with this request and with none: FP32 D2Q37 363 / 98.2 / 26.1 and
+// 372 / 101.6 / 28.2 (5), D2Q25 247 / 67.9 / 16.5 and 254 / 73.7 / 21.2 (7),
+// D2Q17 178 / 49.1 / 10.6 and 178 / 49.6 / 11.4 (7); BF16DEV D2Q37 293 / 83.9 /
+// 24.2 and 392 / 111.5 / 28.1 (6), D2Q25 249 / 72.0 / 20.5 and 361 / 102.4 / 23.1
+// (6), D2Q17 equal (7); BF16SHIFT D2Q37 236 / 69.0 / 19.3 and 307 / 87.6 / 21.8 (7),
+// D2Q25 194 / 56.0 / 15.1 and 224 / 65.2 / 18.0 (7), D2Q17 equal (7).  FP64 is bound
+// by its FP64 instructions: none is best throughout.
+template <int Q, int PREC>
+constexpr int default_blocks() {
+    if (PREC == LBM_FP64) return 0;
+    if (PREC == LBM_FP32) return Q == 37 ? 5 : 7;
+    if (PREC == LBM_BF16DEV) return Q == 17 ? 7 : 6;
+    return 7;
+}
 
 template <int Q, int PREC, int BX, int MINB, bool CS, int RS>
 int launch_direct(SolverImpl &s, int src, int dst) {
@@ -74,23 +90,34 @@ int launch_direct(SolverImpl &s, int src, int dst) {
     S *fout = (S *)s.f[dst];
     const float *rin = s.rho[src];
     float *rout = s.rho[dst];
-    // a pitch class: offsets as instruction immediates (compiled for the
-    // 37-velocity lattice; the others take the offsets from the constants)
-    if constexpr (Q == 37 && BX == 128 && RS == 1) {
-        constexpr int P0 = pitch_class(PREC, 0), P1 = pitch_class(PREC, 1),
-                      P2 = pitch_class(PREC, 2);
-        if (k.pitch == P0)
-            return (int)cudaLaunchKernelEx(&cfg, k_step_direct<Q, PREC, BX, MINB, CS, RS, P0>, fin,
-                                           fout, rin, rout, k, s.kw);
-        if (k.pitch == P1)
-            return (int)cudaLaunchKernelEx(&cfg, k_step_direct<Q, PREC, BX, MINB, CS, RS, P1>, fin,
-                                           fout, rin, rout, k, s.kw);
-        if (k.pitch == P2)
-            return (int)cudaLaunchKernelEx(&cfg, k_step_direct<Q, PREC, BX, MINB, CS, RS, P2>, fin,
-                                           fout, rin, rout, k, s.kw);
-    }
-    return (int)cudaLaunchKernelEx(&cfg, k_step_direct<Q, PREC, BX, MINB, CS, RS, 0>, fin, fout, rin,
-                                   rout, k, s.kw);
+    auto go = [&](auto pc, auto iso2) {
+        return (int)cudaLaunchKernelEx(
+            &cfg, k_step_direct<Q, PREC, BX, MINB, CS, RS, decltype(pc)::value, decltype(iso2)::value>,
+            fin, fout, rin, rout, k, s.kw);
+    };
+    // a pitch class: offsets as instruction immediates, else from the
+    // constants; compiled for the one-row 128-column shapes of the 37-velocity
+    // lattice and, for the others, for variant 0's
+    auto by_pitch = [&](auto iso2) {
+        if constexpr (BX == 128 && RS == 1 &&
+                      (Q == 37 || (MINB == default_blocks<Q, PREC>() && !CS))) {
+            constexpr int P0 = pitch_class(PREC, 0), P1 = pitch_class(PREC, 1),
+                          P2 = pitch_class(PREC, 2);
+            if (k.pitch == P0) return go(std::integral_constant<int, P0>{}, iso2);
+            if (k.pitch == P1) return go(std::integral_constant<int, P1>{}, iso2);
+            if (k.pitch == P2) return go(std::integral_constant<int, P2>{}, iso2);
+        }
+        return go(std::integral_constant<int, 0>{}, iso2);
+    };
+    // variant 0's shape also with the second-order isothermal equilibrium of the
+    // 17- and 25-velocity lattices compiled in, us per step on 2050 x 1023 with
+    // and without (the pitch in both): D2Q25 FP32 66.7 and 67.9, BF16DEV 57.7 and
+    // 72.0, BF16SHIFT 48.1 and 56.0, FP64 792 and 1026; D2Q17 46.3 / 49.1, 43.0 / 50.0,
+    // 38.7 / 45.2, 569 / 743.  (The fourth-order thermal one compiled in gained
+    // nothing on D2Q37: FP32 366.7 against 363, BF16SHIFT 246 against 236.)
+    if constexpr (Q != 37 && BX == 128 && RS == 1 && !CS && MINB == default_blocks<Q, PREC>())
+        if (k.eq_order == 2 && !k.thermal && !k.const_tau) return by_pitch(std::true_type{});
+    return by_pitch(std::false_type{});
 }
 
 // One lattice's direct-kernel variants (the 37-velocity ones, with their
@@ -100,8 +127,9 @@ int step_q(SolverImpl &s, int src, int dst, int variant) {
     using V = DirectVariants;
 #define LBM_DIRECT_CASE(I)                                                                  \
     case I:                                                                                 \
-        return launch_direct<Q, PREC, V::v[I][0], V::v[I][1], (V::v[I][2] != 0), V::v[I][3]>( \
-            s, src, dst);
+        return launch_direct<Q, PREC, V::v[I][0],                                           \
+                             (V::v[I][1] < 0 ? default_blocks<Q, PREC>() : V::v[I][1]),     \
+                             (V::v[I][2] != 0), V::v[I][3]>(s, src, dst);
     switch (variant) {
         LBM_DIRECT_CASE(0)
         LBM_DIRECT_CASE(1)

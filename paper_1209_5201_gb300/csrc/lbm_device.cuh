@@ -389,8 +389,12 @@ struct PairLoop {
 // steady state by about that relative amount.  FP64 keeps the form
 // (1 - omega) f~ + omega rho g.
 //
+// ISO2: the second-order isothermal equilibrium compiled in, without the terms
+// that are zero and the factors that are one (the same results bit for bit on
+// finite states); otherwise the solve's order and thermal flag.
+//
 // V: float or double.
-template <int Q, class V, bool SHIFT = false>
+template <int Q, class V, bool SHIFT = false, bool ISO2 = false>
 struct Collision {
     using L = Lat<Q>;
     using O = Ar<V>;
@@ -426,7 +430,7 @@ struct Collision {
         const V uy = O::mul(O::mul(O::bc(k.r), jy), inv);
         const V u2 = O::fma(ux, ux, O::mul(uy, uy));
         V th = O::bc(C(0)), T = O::bc(C(1));
-        if (k.thermal) {
+        if (!ISO2 && k.thermal) {
             V e2 = O::bc(C(0));
 #pragma unroll
             for (int a = 1; a < Q; a += 2)
@@ -445,9 +449,13 @@ struct Collision {
             }
         }
         V taul;
-        if (k.const_tau) taul = O::bc(k.tau_lat);
-        else if (k.mu_is_one || !k.thermal) taul = O::mul(O::bc(k.K), inv);
-        else taul = O::mul(O::mul(O::bc(k.K), inv), O::pw(T, k.mu_m1));
+        if constexpr (ISO2) {                // no constant tau
+            taul = O::mul(O::bc(k.K), inv);
+        } else {
+            if (k.const_tau) taul = O::bc(k.tau_lat);
+            else if (k.mu_is_one || !k.thermal) taul = O::mul(O::bc(k.K), inv);
+            else taul = O::mul(O::mul(O::bc(k.K), inv), O::pw(T, k.mu_m1));
+        }
         set_omega(O::rcp(O::add(taul, O::bc(C(0.5)))));
         sx = O::mul(O::bc(k.r), ux);
         sy = O::mul(O::bc(k.r), uy);
@@ -467,6 +475,10 @@ struct Collision {
     // the c2-independent factors a00, a01, a02, a10, a11, a20, a21 (and A3, A4)
     __device__ __forceinline__ void powers(V u2, V th, V drr, const KConsts<C> &k, V (&p)[8]) {
         const bool o3 = k.eq_order >= 3, o4 = k.eq_order >= 4;
+        if constexpr (ISO2) {
+            p[0] = O::fma(O::bc(C(-0.5)), u2, SHIFT ? drr : O::bc(C(1)));
+            return;
+        }
         V a00 = O::sub(O::fma(O::bc(C(-0.5)), u2, SHIFT ? drr : O::bc(C(1))), th);
         V a01 = O::mul(O::bc(C(0.5)), th), a02 = O::bc(C(0));
         V a10 = O::bc(C(1)), a11 = O::bc(C(0)), a20 = O::bc(C(0.5)), a21 = O::bc(C(0));
@@ -492,6 +504,11 @@ struct Collision {
     // the coefficients of shell s
     __device__ __forceinline__ static void shell(const V (&p)[8], V orho, const KConsts<C> &k, int s,
                                                  V &A0s, V &A1s, V &A2s, V &cws) {
+        if constexpr (ISO2) {   // A0 alone; A1 = 1, A2 = 1/2, A3 = A4 = 0
+            A0s = p[0];
+            cws = O::mul(orho, O::bc(k.wsh[s]));
+            return;
+        }
         const V c2 = O::bc(k.c2sh[s]);
         A0s = O::fma(O::fma(p[2], c2, p[1]), c2, p[0]);
         A1s = O::fma(p[4], c2, p[3]);
@@ -523,8 +540,14 @@ struct Collision {
         constexpr int s = L::sh(A);
         const V sv = s_of<A>();
         const V s2 = O::mul(sv, sv);
-        const V E = O::fma(s2, O::fma(A4, s2, A2[s]), A0[s]);
-        const V Od = O::mul(sv, O::fma(A3, s2, A1[s]));
+        V E, Od;
+        if constexpr (ISO2) {
+            E = O::fma(s2, O::bc(C(0.5)), A0[s]);
+            Od = sv;
+        } else {
+            E = O::fma(s2, O::fma(A4, s2, A2[s]), A0[s]);
+            Od = O::mul(sv, O::fma(A3, s2, A1[s]));
+        }
         P = O::mul(cw[s], E);
         R = O::mul(cw[s], Od);
     }
