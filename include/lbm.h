@@ -440,8 +440,9 @@ typedef struct lbm_server_cfg {
                                 a cluster (>= 32; default 256): smaller gives
                                 lower latency per request, larger more solves
                                 per second when the GPU is full             */
-    int32_t class_sub[5];    /* chunks per launch of a slot on a cluster of 1,
-                                2, 4, 8, 16 CTAs (0..16; 0: the built-in rule
+    int32_t class_sub[5];    /* chunks every launch runs for a slot on a cluster
+                                of 1, 2, 4, 8, 16 CTAs, more following while they
+                                fit its time (0..16; 0: the built-in rule
                                 max(1, CL / 2)); a cluster runs a step faster
                                 than one CTA, so it runs several chunks while
                                 one-CTA slots run one.  lbm_server_autotune

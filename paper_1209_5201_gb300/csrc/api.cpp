@@ -300,11 +300,7 @@ void fill_wall(KWall &kw, const LatticeHost &L, const lbm_params &p, const KCons
             const int a = kw.out_a[w][l];
             const double c = k.wcoef[w][a];
             const double c0 = shifted ? std::fma(kw.wsum[w], c, -(double)k.w[a]) : 0.0;
-            KWall::Emit &e = kw.e[w][l];
-            e.ch = (float)c;
-            e.cl = (float)(c - (double)e.ch);
-            e.c0h = (float)c0;
-            e.c0l = (float)(c0 - (double)e.c0h);
+            kw.e[w][l] = wall_emit(c, c0);
         }
     }
 }

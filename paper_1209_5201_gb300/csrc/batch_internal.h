@@ -17,8 +17,15 @@ constexpr int kSlotCancelled = 6;         // set by the host; the kernel skips t
 
 // Most velocities leaving one wall (e.n > 0): 15 for D2Q37.
 constexpr int kMaxOut = 16;
-// Most chunks one launch runs for one slot.
+// Most incoming terms per wall: 26 for D2Q37.
+constexpr int kMaxTerm = 28;
+// Chunks one launch runs for one slot: at most kMaxSub for certain (SlotDesc::
+// sub), and more, up to kMaxLaunchChunks, while they fit the launch's time.
 constexpr int kMaxSub = 16;
+constexpr int kMaxLaunchChunks = 256;
+// A launch lasts as long as its slowest slot, at least about this (ns): the
+// host's work per launch is 20 - 50 us.
+constexpr unsigned long long kMinLaunchNs = 2000000ull;
 // Chunks per launch of a slot on a cluster of cl CTAs: about the factor by
 // which the cluster shortens a step of a tall column, conservatively, so that
 // a cluster slot is rarely the one a launch waits for.
@@ -31,8 +38,9 @@ struct SlotDesc {
     int check_every;          // residual every check_every chunks
     int chunk_steps;          // steps this slot runs per chunk launch
     int cl;                   // CTAs of the slot's cluster: 1, 2, 4, 8 or 16
-    int sub;                  // chunks per launch (a cluster runs several, so
-                              // that it keeps pace with one-CTA slots' launches)
+    int sub;                  // chunks every launch runs (a cluster several, so that
+                              // it keeps pace with one-CTA slots' launches); more
+                              // follow while they fit the launch's time
     long long f_off;          // element offset of buffer 0 in the pool
     long long prev_off;       // element offset of the previous-check u_x, T
     double tol;               // target of the extrapolated distance to steady state
@@ -47,14 +55,16 @@ struct SlotDesc {
     // incoming terms of Eq. (12)'s numerator, built on the host: wall w (0
     // bottom, 1 top), term l < nterm is velocity term_a[w][l] at distance
     // term_row[w][l] from the wall
-    int nterm;                // < 32: lane nterm of the wall warp carries wterm
+    int nterm;                // <= kMaxTerm
     int nout;                 // outgoing velocities per wall (e.n > 0), <= kMaxOut
     signed char term_a[2][32];
     signed char term_row[2][32];
+    signed char term_ey[2][32];   // its e_y
     signed char out_a[2][kMaxOut];
-    double wterm[2];          // sum over the incoming terms of their weights w_a
-    double out_c[2][kMaxOut]; // g^w_a / D_w of outgoing velocity out_a[w][l]
-    double out_w[2][kMaxOut]; // its weight w_a as the FP32 storage holds it
+    // its re-emission M_in g^w_a / D_w - w_a = c0 + d c with d the sum of the
+    // incoming deviations, c = g^w_a / D_w and c0 = (the terms' weights) c - w_a,
+    // both as pairs of floats
+    KWall::Emit out_e[2][kMaxOut];
     KConsts<float> k;         // per-instance constants (Nx = 1, pitch = 1)
 };
 
@@ -70,6 +80,8 @@ struct SlotStatus {
     int checks;
     int since_best;           // checks without a new smallest residual
     int chunks;               // chunks run since admission
+    long long first_ns;       // time the last launch's d.sub chunks took
+    int go;                   // another chunk in this launch (shared by the cluster)
     int precise;              // 0: round-to-nearest collision; 1: conserving
                               // increments with stochastic rounding (2: switching)
 };
@@ -113,12 +125,12 @@ int preload_batch_kernels();
 int batch_max_cluster();
 // dbg: 8 device ints; dbg[0] != 0 records the first invalid descriptor or
 // read-out offset a kernel met (and skipped).
-// One chunk of the slots [slot0, slot0 + nlanes), each on a cluster of CL
-// CTAs; part: kMaxResidualChunks x 6 FP64 residual partials per slot of the
+// Chunks of the slots [slot0, slot0 + nlanes), each on a cluster of CL CTAs;
+// budget: device word with the time (ns) the launch may take anyway; part: kMaxResidualChunks x 6 FP64 residual partials per slot of the
 // whole table.
 int launch_batch_chunk(cudaStream_t st, SlotDesc *desc, SlotStatus *status, float *pool,
                        double *part, int slot0, int nlanes, int CL, long long pool_elems,
-                       int *dbg);
+                       const unsigned long long *budget, int *dbg);
 int launch_batch_init(cudaStream_t st, SlotDesc *desc, float *pool, const int *slots, int n,
                       float rho0, int nslots, long long pool_elems, int *dbg);
 int launch_batch_macros(cudaStream_t st, const SlotDesc *desc, const float *pool,

@@ -15,11 +15,12 @@ __device__ __forceinline__ bool desc_ok(const SlotDesc &d, long long pool_elems,
                                         int code, int *dbg) {
     const bool q_ok = d.Q == 17 || d.Q == 25 || d.Q == 37;
     const long long need = 2LL * d.Q * d.Ny + 2LL * d.Ny;
-    bool terms_ok = d.nterm >= 1 && d.nterm < 32 && d.nout >= 1 && d.nout <= kMaxOut;
+    bool terms_ok = d.nterm >= 1 && d.nterm <= kMaxTerm && d.nout >= 1 && d.nout <= kMaxOut;
     for (int w = 0; w < 2 && terms_ok; ++w) {
         for (int l = 0; l < d.nterm; ++l)
             terms_ok = terms_ok && d.term_a[w][l] >= 0 && d.term_a[w][l] < d.Q &&
-                       d.term_row[w][l] >= 0 && d.term_row[w][l] < 3;
+                       d.term_row[w][l] >= 0 && d.term_row[w][l] < 3 &&
+                       d.term_ey[w][l] >= -3 && d.term_ey[w][l] <= 3;
         for (int l = 0; l < d.nout; ++l)
             terms_ok = terms_ok && d.out_a[w][l] >= 0 && d.out_a[w][l] < d.Q;
     }
@@ -52,14 +53,15 @@ __device__ __forceinline__ void load_desc(const SlotDesc *g, SlotDesc *s) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
 }
 
-// One chunk of slot slot0 + blockIdx.x / CL on a cluster of CL CTAs (CL = 1:
+// Chunks of slot slot0 + blockIdx.x / CL on a cluster of CL CTAs (CL = 1:
 // a plain launch).  Every CTA of a cluster reads the same descriptor and
 // status, so all of them take the same early exit or none does: no thread
 // leaves while others of its cluster still meet barriers.
 __global__ void __launch_bounds__(kBatchThreads, 2)
 k_batch_chunk(SlotDesc *__restrict__ desc, SlotStatus *__restrict__ status,
               float *__restrict__ pool, double *__restrict__ part, int slot0, int CL,
-              long long pool_elems, int *dbg) {
+              long long pool_elems, const unsigned long long *__restrict__ budget, int *dbg) {
+    const unsigned long long t0 = global_ns();
     __shared__ SlotDesc sd;
     __shared__ BatchWallShared sw;
     __shared__ int s_chunks, s_precise;
@@ -79,14 +81,14 @@ k_batch_chunk(SlotDesc *__restrict__ desc, SlotStatus *__restrict__ status,
     double *pp = part + (long long)slot * (6 * kMaxResidualChunks);
     int done = 0;
     switch (sd.Q) {
-    case 17: done = batch_slot<17>(sd, pool, status + slot, sw, rank, CL, s_chunks, s_steps, s_precise, pp, batch_sm); break;
-    case 25: done = batch_slot<25>(sd, pool, status + slot, sw, rank, CL, s_chunks, s_steps, s_precise, pp, batch_sm); break;
-    case 37: done = batch_slot<37>(sd, pool, status + slot, sw, rank, CL, s_chunks, s_steps, s_precise, pp, batch_sm); break;
+    case 17: done = batch_slot<17>(sd, pool, status + slot, sw, rank, CL, s_chunks, s_steps, s_precise, pp, batch_sm, t0, *budget); break;
+    case 25: done = batch_slot<25>(sd, pool, status + slot, sw, rank, CL, s_chunks, s_steps, s_precise, pp, batch_sm, t0, *budget); break;
+    case 37: done = batch_slot<37>(sd, pool, status + slot, sw, rank, CL, s_chunks, s_steps, s_precise, pp, batch_sm, t0, *budget); break;
     default: break;
     }
     // the global-memory path leaves the state in the other buffer after an odd
     // number of steps; the shared-memory path writes it back where it came from
-    const bool smem = batch_uses_smem(sd.Ny, CL);
+    const bool smem = batch_uses_smem(sd.Ny, CL, sd.k.accom[0] == 1.0 && sd.k.accom[1] == 1.0);
     if (!smem && rank == 0 && threadIdx.x == 0)
         desc[slot].cur = (int)((sd.cur + (long long)done * sd.chunk_steps) & 1);
 }
@@ -225,11 +227,11 @@ int batch_max_cluster() {
 
 int launch_batch_chunk(cudaStream_t st, SlotDesc *desc, SlotStatus *status, float *pool,
                        double *part, int slot0, int nlanes, int CL, long long pool_elems,
-                       int *dbg) {
+                       const unsigned long long *budget, int *dbg) {
     if (nlanes <= 0) return 0;
     if (CL == 1) {
         k_batch_chunk<<<nlanes, kBatchThreads, kSmemBytes, st>>>(desc, status, pool, part, slot0,
-                                                                 1, pool_elems, dbg);
+                                                                 1, pool_elems, budget, dbg);
         return (int)cudaGetLastError();
     }
     if (CL != 2 && CL != 4 && CL != 8 && CL != 16) return (int)cudaErrorInvalidValue;
@@ -246,7 +248,7 @@ int launch_batch_chunk(cudaStream_t st, SlotDesc *desc, SlotStatus *status, floa
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return (int)cudaLaunchKernelEx(&cfg, k_batch_chunk, desc, status, pool, part, slot0, CL,
-                                   pool_elems, dbg);
+                                   pool_elems, budget, dbg);
 }
 
 int launch_batch_init(cudaStream_t st, SlotDesc *desc, float *pool, const int *slots, int n,

@@ -8,20 +8,20 @@
 // f~*(j - e_ay, a).  A slot runs on a cluster of CL CTAs (CL = 1, 2, 4, 8 or
 // 16, fixed by its height): CTA `rank` owns rows [rank R, rank R + R), R =
 // ceil(Ny / CL), and a cluster barrier with release / acquire semantics
-// separates the steps.  When R <= kSmemRows the CTA keeps its rows' two state
-// buffers in shared memory for the whole launch (loaded from the pool at the
-// start, written back at the end; rows of Q populations) and pulls the <= 3
-// rows it needs from each neighbour through distributed shared memory
-// (ld.shared::cluster); taller blocks keep the state in global memory
-// (L2-resident) and read it with ld.global.cg.
+// separates the steps.  When its rows fit (batch_uses_smem) the CTA keeps them in shared
+// memory for the whole launch (loaded from the pool at the start, written back
+// at the end; one ring per velocity, SmemState) and pulls the <= 3 rows it needs
+// from each neighbour through distributed shared memory (ld.shared::cluster);
+// taller blocks keep the state in global memory (L2-resident, two buffers) and
+// read it with ld.global.cg.
 //
 // Row mapping inside a CTA: warp 0 of the bottom CTA owns the (up to) 32
-// lowest rows and warp 1 of the top CTA the 32 highest; each of those warps
-// first sums its wall's incoming mass (numerator of Eq. (12)) in FP64 by a
-// warp shuffle in a fixed lane order - lane l loads the l-th (velocity, row)
-// term of the wall's list, built on the host and carried in the slot
-// descriptor - forms the normalised re-emission of every outgoing velocity
-// once, and then updates its rows (branch-free: sources clamped into the
+// lowest rows and warp 0 (one CTA: warp 1) of the top CTA the 32 highest; each of
+// those warps first sums its wall's incoming mass (numerator of Eq. (12)) to
+// FP64 precision in a fixed order - the (velocity, row) terms of the wall's
+// list, built on the host and carried in the slot descriptor - forms the
+// normalised re-emission of every outgoing velocity once, and then updates its
+// rows (branch-free: sources clamped into the
 // slot, the wall's values selected afterwards).  The other rows never need a wall value,
 // so no block barrier separates the wall sums from the bulk update.  Every
 // slot's arithmetic depends only on the slot itself (its cluster size is a
@@ -42,6 +42,7 @@ struct BatchWallShared {
     float fill[2][kMaxQ];
     float acc[2];
     float term[2][3][kMaxQ];
+    int toff[2][kMaxTerm];     // where a state keeps each incoming term (its term_at)
 };
 
 __device__ __forceinline__ unsigned cluster_rank() {
@@ -70,13 +71,14 @@ __device__ __forceinline__ void slot_barrier(int CL) {
     cluster_wait();
 }
 
-// Rows of a CTA's shared-memory state: two buffers of Q x kSmemRows floats.
-constexpr int kSmemRows = 256;
-constexpr int kSmemBytes = 2 * kMaxQ * kSmemRows * (int)sizeof(float);
+// Slots of a CTA's shared-memory state (SmemState).
+constexpr int kRing = 512;
+constexpr int kSmemBytes = kMaxQ * kRing * (int)sizeof(float);
 
-// The shared-memory path serves every column whose CTAs' rows fit.
-__host__ __device__ inline bool batch_uses_smem(int Ny, int CL) {
-    return batch_rows_per_cta(Ny, CL) <= kSmemRows;
+// The shared-memory path serves every column whose CTAs' rows fit: three slots
+// fewer than the ring has, or all of them on one CTA between diffuse walls.
+__host__ __device__ inline bool batch_uses_smem(int Ny, int CL, bool diffuse) {
+    return batch_rows_per_cta(Ny, CL) <= (CL == 1 && diffuse ? kRing : kRing - 3);
 }
 
 // Population a of the wall re-emission (Eq. (9) with R = accom R_D + (1 -
@@ -112,7 +114,7 @@ __device__ __forceinline__ void apply_walls(const BatchWallShared &sw, int j, in
         for (int a = 0; a < Q; ++a) {
             const int sj = j - L::ey(a);
             if (sj < 0 || sj >= Ny)
-                f[a] = wall_value(sw, sj < 0 ? 0 : 1, a, [&] { return mirror(a); });
+                f[a] = wall_value(sw, sj < 0 ? 0 : 1, a, [&] { return mirror(a, L::ey(a)); });
         }
     }
 }
@@ -120,6 +122,7 @@ __device__ __forceinline__ void apply_walls(const BatchWallShared &sw, int j, in
 // Slot state in global memory (pool), two buffers of [Q][Ny]; a step reads
 // `src` and writes `dst`, rows of any CTA of the cluster.
 struct GlobalState {
+    static constexpr bool kTwoBuffers = false;   // (of shared memory)
     const float *src;
     float *dst;
     int Ny;
@@ -129,11 +132,10 @@ struct GlobalState {
     __device__ __forceinline__ float ld(int a, int row) const {
         return __ldcg(src + (long long)a * Ny + row);
     }
-    __device__ __forceinline__ float ld_own(int a, int row) const { return ld(a, row); }
+    __device__ __forceinline__ float ld_at(int a, int, int row) const { return ld(a, row); }
     // wall w's incoming term (a, kk) of the step just done (staged by store)
-    __device__ __forceinline__ float term(int w, int a, int kk, int) const {
-        return stage[(w * 3 + kk) * kMaxQ + a];
-    }
+    __device__ __forceinline__ int term_off(int w, int a, int, int kk) const { return (w * 3 + kk) * kMaxQ + a; }
+    __device__ __forceinline__ float term_at(int off) const { return stage[off]; }
     // f_in of row j (Eq. (5) pull with the Eq. (12) wall)
     template <int Q, bool EDGE>
     __device__ __forceinline__ void pull(const SlotDesc &d, const BatchWallShared &sw, int j,
@@ -144,26 +146,24 @@ struct GlobalState {
             const int sj = j - L::ey(a);
             f[a] = ld(a, EDGE ? min(max(sj, 0), Ny - 1) : sj);
         }
-        if constexpr (EDGE) apply_walls<Q>(sw, j, Ny, f, [&](int a) { return ld(d.k.mirror[a], j); });
+        if constexpr (EDGE) apply_walls<Q>(sw, j, Ny, f, [&](int a, int) { return ld(d.k.mirror[a], j); });
     }
-    template <int Q, bool EDGE>
+    template <int Q>
     __device__ __forceinline__ void store(int j, const float (&o)[Q]) const {
         using L = Lat<Q>;
 #pragma unroll
         for (int a = 0; a < Q; ++a) dst[(long long)a * Ny + j] = o[a];
-        if constexpr (EDGE) {
-            // the velocities that stream into a wall from its 3 nearest rows
-            if (j < 3) {
-                StaticFor<0, Q>::run([&](auto ic) {
-                    constexpr int a = decltype(ic)::value;
-                    if constexpr (L::ey(a) < 0) stage[j * kMaxQ + a] = o[a];
-                });
-            } else if (j >= Ny - 3) {
-                StaticFor<0, Q>::run([&](auto ic) {
-                    constexpr int a = decltype(ic)::value;
-                    if constexpr (L::ey(a) > 0) stage[(3 + Ny - 1 - j) * kMaxQ + a] = o[a];
-                });
-            }
+        // the velocities that stream into a wall from its 3 nearest rows
+        if (j < 3) {
+            StaticFor<0, Q>::run([&](auto ic) {
+                constexpr int a = decltype(ic)::value;
+                if constexpr (L::ey(a) < 0) stage[j * kMaxQ + a] = o[a];
+            });
+        } else if (j >= Ny - 3) {
+            StaticFor<0, Q>::run([&](auto ic) {
+                constexpr int a = decltype(ic)::value;
+                if constexpr (L::ey(a) > 0) stage[(3 + Ny - 1 - j) * kMaxQ + a] = o[a];
+            });
         }
     }
     __device__ __forceinline__ void flip() {
@@ -192,9 +192,10 @@ __device__ __forceinline__ void sts_f32(uint32_t addr, float v) {
 // shared memory), without a compiler memory clobber: ordered only against the
 // other volatile asm (the loads, stores and barriers of this file), so the
 // constants read around it can stay in registers.
+template <int OFF>
 __device__ __forceinline__ float ldsc_f32_nc(uint32_t addr) {
     float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(v) : "r"(addr));
+    asm volatile("ld.shared::cluster.f32 %0, [%1+%2];\n" : "=f"(v) : "r"(addr), "n"(OFF));
     return v;
 }
 // shared::cluster address of the same location in CTA `rank` of the cluster
@@ -204,93 +205,165 @@ __device__ __forceinline__ uint32_t map_rank(uint32_t addr, unsigned rank) {
     return out;
 }
 
-// Slot state in the cluster's shared memory.  This CTA holds rows [j0, j0 + R)
-// in two buffers of R rows x Q floats (row-major: a thread's Q populations are
-// contiguous and Q is odd, so the 32 lanes of a warp, on 32 consecutive rows,
-// hit 32 different banks); `b` is the buffer holding the current state.  lo /
-// hi are the same buffers of the neighbouring CTAs (rows j0 - R .., j0 + R ..)
-// as shared::cluster addresses, 0 at the slot's ends.  Bulk rows read with
-// compile-time offsets from their own row address.
-template <int Q>
+// Slot state in the cluster's shared memory: rows of Q floats (row-major: a
+// thread's Q populations are contiguous and Q is odd, so the 32 lanes of a warp,
+// on 32 consecutive rows, hit 32 different banks).  lo / hi are the neighbours'
+// shared memory (rows below / above) as shared::cluster addresses, 0 at the
+// slot's ends.
+//  * Two buffers of up to kRing / 2 rows (RING false): slot lr of a buffer is
+//    local row lr; bulk rows read with compile-time offsets.
+//  * One buffer of up to kRing rows (RING): every velocity is a ring that turns
+//    by its e_y slots per step: after t steps of the launch local row lr is at slot
+//    (lr - t e_y) mod kRing, so the value a row pulls and the value it stores for
+//    that velocity share one slot, no other row touches it, and a step needs no
+//    second buffer.  304 columns of 512 rows: 5.2 us per step, 6.45 with the
+//    state in L2, whose bandwidth bounds a full GPU there; the slots' address
+//    arithmetic costs 6 % where two buffers fit (a lone 128-row column 1.41 and
+//    1.33 us).  What leaves a CTA stays readable in its slots during the step in
+//    which what enters it is stored, if the ring has three slots beyond the rows
+//    (a neighbour reads it then); on one CTA only its own walls read it, before
+//    the step's barrier.
+template <int Q, bool RING>
 struct SmemState {
-    uint32_t base;             // shared::cta address of buffer 0
-    uint32_t lo, hi;           // shared::cluster addresses of the neighbours' buffer 0
-    uint32_t self;             // shared::cluster address of this CTA's buffer 0
-    int R, j0, b;
-    __device__ __forceinline__ uint32_t row_addr(int buf, int lr) const {
-        return base + (uint32_t)((buf * R + lr) * Q) * 4u;
+    static constexpr bool kTwoBuffers = !RING;
+    uint32_t base;             // shared::cta address
+    uint32_t lo, hi;           // shared::cluster addresses of the neighbours
+    uint32_t self;             // shared::cluster address of this CTA
+    int rpc, j0, Ny;           // rows per CTA, first row, rows of the slot
+    int t;                     // RING: steps since the launch began; else: current buffer
+    // slot of local row lr for a velocity of vertical component e, now
+    __device__ __forceinline__ int slot_of(int lr, int e) const {
+        if constexpr (RING) return (lr - e * t) & (kRing - 1);
+        else return t * (kRing / 2) + lr;
     }
-    __device__ __forceinline__ float ld_own(int a, int row) const {
-        return lds_f32(row_addr(b, row - j0) + (uint32_t)a * 4u);
+    __device__ __forceinline__ uint32_t slot_addr(int sl) const { return base + (uint32_t)(sl * Q) * 4u; }
+    __device__ __forceinline__ void flip() {
+        if constexpr (RING) ++t;
+        else t ^= 1;
     }
-    // wall w's incoming term (a, kk): row kk from the wall of the current state
-    __device__ __forceinline__ float term(int w, int a, int kk, int Ny) const {
-        return ld_own(a, w == 0 ? kk : Ny - 1 - kk);
+    // population a (vertical component e) of slot row `row` of this CTA, now
+    __device__ __forceinline__ float ld_at(int a, int e, int row) const {
+        return lds_f32(slot_addr(slot_of(row - j0, e)) + (uint32_t)a * 4u);
+    }
+    // wall w's incoming term (a, kk), row kk from the wall of the current state:
+    // local row, velocity and e_y packed
+    __device__ __forceinline__ int term_off(int w, int a, int e, int kk) const {
+        return ((w == 0 ? kk : Ny - 1 - kk) - j0) | (a << 16) | ((e + 4) << 24);
+    }
+    __device__ __forceinline__ float term_at(int off) const {
+        return lds_f32(slot_addr(slot_of(off & 0xffff, (off >> 24) - 4)) + (uint32_t)((off >> 16) & 0xff) * 4u);
     }
     template <int Q_, bool EDGE>
     __device__ __forceinline__ void pull(const SlotDesc &d, const BatchWallShared &sw, int j,
                                          float (&f)[Q_]) const {
         using L = Lat<Q_>;
-        if constexpr (!EDGE) {
-            // every source row lies in [lr - 3, lr + 3] of this CTA: offsets
-            // from row lr - 3 are compile-time constants
-            const uint32_t r0 = row_addr(b, j - j0 - 3);
+        if constexpr (!EDGE && !RING) {
+            // every source row is one of this CTA's: offsets from row lr - 3
+            const uint32_t r0 = slot_addr(slot_of(j - j0 - 3, 0));
             StaticFor<0, Q_>::run([&](auto ic) {
                 constexpr int a = decltype(ic)::value;
                 f[a] = lds_f32<((3 - L::ey(a)) * Q_ + a) * 4>(r0);
+            });
+            return;
+        }
+        uint32_t r[7];
+        if constexpr (!EDGE) {
+            StaticFor<0, 7>::run([&](auto ic) {
+                constexpr int e = decltype(ic)::value - 3;
+                r[e + 3] = slot_addr(slot_of(j - j0 - e, e));
+            });
+            StaticFor<0, Q_>::run([&](auto ic) {
+                constexpr int a = decltype(ic)::value;
+                f[a] = lds_f32<a * 4>(r[L::ey(a) + 3]);
             });
         } else {
             // source row clamped into the slot, then into this CTA or a
             // neighbour (selects, no branch): every load goes through the
             // shared::cluster window and all of them issue back to back
-#pragma unroll
-            for (int a = 0; a < Q_; ++a) {
-                const int lr = min(max(j - L::ey(a), 0), d.Ny - 1) - j0;
-                const uint32_t bse = lr < 0 ? lo : (lr >= R ? hi : self);
-                const int rr = lr < 0 ? lr + R : (lr >= R ? lr - R : lr);
-                f[a] = ldsc_f32_nc(bse + (uint32_t)(((b * R + rr) * Q_ + a) * 4));
-            }
-            apply_walls<Q_>(sw, j, d.Ny, f, [&](int a) { return ld_own(d.k.mirror[a], j); });
+            StaticFor<0, 7>::run([&](auto ic) {
+                constexpr int e = decltype(ic)::value - 3;
+                const int l = min(max(j - e, 0), d.Ny - 1) - j0;
+                const uint32_t bse = l < 0 ? lo : (l >= rpc ? hi : self);
+                const int ln = l < 0 ? l + rpc : (l >= rpc ? l - rpc : l);
+                r[e + 3] = bse + (uint32_t)(slot_of(ln, e) * Q) * 4u;
+            });
+            StaticFor<0, Q_>::run([&](auto ic) {
+                constexpr int a = decltype(ic)::value;
+                f[a] = ldsc_f32_nc<a * 4>(r[L::ey(a) + 3]);
+            });
+            apply_walls<Q_>(sw, j, d.Ny, f, [&](int a, int e) { return ld_at(d.k.mirror[a], -e, j); });
         }
     }
-    template <int Q_, bool EDGE>
+    template <int Q_>
     __device__ __forceinline__ void store(int j, const float (&o)[Q_]) const {
-        const uint32_t r = row_addr(b ^ 1, j - j0);
-        StaticFor<0, Q_>::run([&](auto ic) {
-            constexpr int a = decltype(ic)::value;
-            sts_f32<a * 4>(r, o[a]);
-        });
+        using L = Lat<Q_>;
+        if constexpr (RING) {
+            uint32_t r[7];
+            StaticFor<0, 7>::run([&](auto ic) {
+                constexpr int e = decltype(ic)::value - 3;
+                r[e + 3] = slot_addr(slot_of(j - j0 - e, e));
+            });
+            StaticFor<0, Q_>::run([&](auto ic) {
+                constexpr int a = decltype(ic)::value;
+                sts_f32<a * 4>(r[L::ey(a) + 3], o[a]);
+            });
+        } else {
+            const uint32_t r = slot_addr((t ^ 1) * (kRing / 2) + j - j0);
+            StaticFor<0, Q_>::run([&](auto ic) {
+                constexpr int a = decltype(ic)::value;
+                sts_f32<a * 4>(r, o[a]);
+            });
+        }
     }
-    __device__ __forceinline__ void flip() { b ^= 1; }
 };
 
-// Numerator of Eq. (12) for `wall` summed by one full warp in FP64, and the
-// normalised re-emission M_in g^w_a / D_w of each outgoing velocity formed
-// once in FP64 (lane l: outgoing velocity out_a[l]) and kept as an FP32
-// deviation from w_a.  Lane l < nterm carries its term's deviation d = f - w,
-// lane nterm the terms' weights summed on the host, so M_in = sum d + sum w;
-// a butterfly of shuffles leaves the same fixed-order sum in every lane.
-// GB300's FP64 rate is a small fraction of its FP32 rate: eight FP64
-// instructions per wall and step, none in the per-cell update.  `term(a, kk)`
-// reads the incoming term (a, kk) of the current state; the wall rows belong
-// to this CTA.
+// Numerator of Eq. (12) for `wall` summed by one full warp, and the normalised
+// re-emission M_in g^w_a / D_w of each outgoing velocity (lane l: out_a[l]), as an
+// FP32 deviation from w_a.  A step is as long as its wall warp: the update of
+// its rows, this, and the barrier.  In FP64 (an add per butterfly stage, the
+// conversions, the product) it took 1200 - 1550 cycles of a lone column's 3300 -
+// 4900 per step, since every FP64 warp instruction takes 64 on GB300.  So the
+// sum of the deviations runs in FP32 with error-free additions (Sum3: to far
+// below FP64's rounding): every group of four lanes sums all terms, seven per
+// lane, then two butterfly stages; and c0 + d c is evaluated in pairs of floats,
+// hi + lo to 2^-46.  terms(t, x) reads the incoming terms t[] of the current state;
+// the wall rows belong to this CTA.
 // The FP32 value of each re-emission is rounded stochastically (add_sr of
 // its round-to-nearest value and the FP32 remainder), from the hash of the
 // step and a counter beyond the slot's rows.
+constexpr int kLaneTerms = kMaxTerm / 4;
 template <class TermFn>
 __device__ __forceinline__ void wall_fill_warp(const SlotDesc &d, int wall, int lane,
-                                               float *fill, uint32_t step, TermFn &&term) {
-    double v = 0.0;
-    if (lane < d.nterm) v = (double)term(d.term_a[wall][lane], d.term_row[wall][lane]);
-    else if (lane == d.nterm) v = d.wterm[wall];
+                                               float *fill, uint32_t step, TermFn &&terms) {
+    const int l = min(lane, d.nout - 1);
+    const KWall::Emit ce = d.out_e[wall][l];
+    // this lane's terms (lane & 3) + 4 i, all loads in flight; past the last
+    // term the loads repeat it
+    float x[kLaneTerms];
+    int t[kLaneTerms];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane < d.nout) {
-        const double x = fma(v, d.out_c[wall][lane], -d.out_w[wall][lane]);
-        const float hi = (float)x, lo = (float)(x - (double)hi);
-        const uint32_t h = sr_cell(step, (uint32_t)(d.Ny + wall));
-        fill[d.out_a[wall][lane]] = add_sr(hi, lo, sr_bits32(h, lane));
+    for (int i = 0; i < kLaneTerms; ++i) t[i] = min((lane & 3) + 4 * i, d.nterm - 1);
+    terms(t, x);
+    Sum3 sum;
+#pragma unroll
+    for (int i = 0; i < kLaneTerms; ++i) sum.add((lane & 3) + 4 * i < d.nterm ? x[i] : 0.0f);
+#pragma unroll
+    for (int o = 1; o <= 2; o <<= 1) {
+        const float h = __shfl_xor_sync(0xffffffffu, sum.h, o), m = __shfl_xor_sync(0xffffffffu, sum.m, o),
+                    r = __shfl_xor_sync(0xffffffffu, sum.l, o);
+        sum.add(h);
+        sum.add(m);
+        sum.l = __fadd_rn(sum.l, r);
     }
+    const float dh = __fadd_rn(sum.h, sum.m);
+    const float dl = __fadd_rn(__fsub_rn(sum.m, __fsub_rn(dh, sum.h)), sum.l);
+    const float p = __fmul_rn(dh, ce.ch), e = __fmaf_rn(dh, ce.ch, -p);
+    float v, r;
+    two_sum(ce.c0h, p, v, r);
+    const float z = __fadd_rn(r, __fadd_rn(ce.c0l, __fmaf_rn(dh, ce.cl, __fmaf_rn(dl, ce.ch, e))));
+    const float hi = __fadd_rn(v, z), lo = __fsub_rn(z, __fsub_rn(hi, v));
+    const uint32_t h = sr_cell(step, (uint32_t)(d.Ny + wall));
+    if (lane < d.nout) fill[d.out_a[wall][l]] = add_sr(hi, lo, sr_bits32(h, lane));
     __syncwarp();
 }
 
@@ -300,8 +373,11 @@ __device__ __forceinline__ void wall_fill_warp(const SlotDesc &d, int wall, int 
 // one of this CTA's rows.
 // PRECISE: conserving increments with stochastic rounding (the steady-state
 // phase of a solve); otherwise the plain relaxation rounded to nearest.
-template <int Q, bool EDGE, bool PRECISE, class State>
-__device__ __forceinline__ void cell_update(const SlotDesc &d, const State &S, int j,
+// The two pulls share one collision and store: a step's loop then holds half the
+// code, which an SM's instruction cache keeps: a lone 128-row D2Q37 column 1.33 us
+// per step, 1.45 with a collision per pull (stochastic 1.78 and 1.83).
+template <int Q, bool PRECISE, class State>
+__device__ __forceinline__ void cell_update(const SlotDesc &d, const State &S, int j, bool edge,
                                             const BatchWallShared &sw, uint32_t step) {
     // the slot's constants live in shared memory; this compiler barrier keeps
     // them there (re-read per cell) instead of hoisted into registers for the
@@ -309,7 +385,8 @@ __device__ __forceinline__ void cell_update(const SlotDesc &d, const State &S, i
     asm volatile("" ::: "memory");
     const KConsts<float> &k = d.k;
     float f[Q];
-    S.template pull<Q, EDGE>(d, sw, j, f);
+    if (edge) S.template pull<Q, true>(d, sw, j, f);
+    else S.template pull<Q, false>(d, sw, j, f);
     Collision<Q, float, true> col;
     col.setup(f, k);
     // PRECISE: increments that conserve mass, momentum (and energy) in FP32,
@@ -326,12 +403,12 @@ __device__ __forceinline__ void cell_update(const SlotDesc &d, const State &S, i
             col.template pair<A>(f[A], f[A + 1], o[A], o[A + 1]);
         });
     }
-    S.template store<Q, EDGE>(j, o);
+    S.template store<Q>(j, o);
 }
 
-// The chunk's time steps.  Warp 0 of the bottom CTA and warp 1 of the top CTA
-// own the wall blocks [j0, j0 + nb) and [j1 - nt, j1) and first form their
-// wall's re-emission; every thread then updates its wall-block row (if any)
+// The chunk's time steps.  Warp 0 of the bottom CTA and warp 0 (one CTA: warp
+// 1) of the top CTA own the wall blocks [j0, j0 + nb) and [j1 - nt, j1) and first
+// form their wall's re-emission; every thread then updates its wall-block row (if any)
 // and its share of the bulk rows [mb, me), handed out from the last thread
 // down so that the wall warps get bulk rows last.
 template <int Q, bool PRECISE, class State>
@@ -340,21 +417,37 @@ __device__ __forceinline__ void run_steps(const SlotDesc &d, State &S, BatchWall
                                           int nth, int j0, int j1, int nb, int nt, int mb,
                                           int me, uint32_t step0) {
     int jw = -1;
+    // the top wall's warp: not the bottom wall's, and none of those that the
+    // bulk rows of a full CTA with one wall fill
+    const int wtop = nb > 0 ? 1 : 0;
     if (warp == 0 && nb > 0 && lane < nb) jw = j0 + lane;
-    if (warp == 1 && nt > 0 && lane < nt) jw = j1 - nt + lane;
+    if (warp == wtop && nt > 0 && lane < nt) jw = j1 - nt + lane;
     const int jb = mb + (nth - 1 - tid);
     // a wall warp's incoming terms are rows of its own wall block
-    const bool wall_warp = (warp == 0 && nb > 0) || (warp == 1 && nt > 0);
-    const int wall = warp == 0 ? 0 : 1;
+    const bool wall_warp = (warp == 0 && nb > 0) || (warp == wtop && nt > 0);
+    const int wall = warp == 0 && nb > 0 ? 0 : 1;
     const int Ny = d.Ny;
     // the chunk's first wall sums read the state as loaded; later ones the
     // wall rows just written (staged in shared memory on the global path)
-    if (wall_warp)
-        wall_fill_warp(d, wall, lane, sw.fill[wall], step0,
-                       [&](int a, int kk) { return S.ld_own(a, wall == 0 ? kk : Ny - 1 - kk); });
+    if (wall_warp) {
+        for (int t = lane; t < d.nterm; t += 32)
+            sw.toff[wall][t] = S.term_off(wall, d.term_a[wall][t], d.term_ey[wall][t], d.term_row[wall][t]);
+        wall_fill_warp(d, wall, lane, sw.fill[wall], step0, [&](const int (&t)[kLaneTerms], float (&x)[kLaneTerms]) {
+#pragma unroll
+            for (int i = 0; i < kLaneTerms; ++i) {
+                const int kk = d.term_row[wall][t[i]];
+                x[i] = S.ld_at(d.term_a[wall][t[i]], d.term_ey[wall][t[i]], wall == 0 ? kk : Ny - 1 - kk);
+            }
+        });
+    }
     auto fill_next = [&](uint32_t st) {
-        wall_fill_warp(d, wall, lane, sw.fill[wall], st,
-                       [&](int a, int kk) { return S.term(wall, a, kk, Ny); });
+        wall_fill_warp(d, wall, lane, sw.fill[wall], st, [&](const int (&t)[kLaneTerms], float (&x)[kLaneTerms]) {
+            int off[kLaneTerms];
+#pragma unroll
+            for (int i = 0; i < kLaneTerms; ++i) off[i] = sw.toff[wall][t[i]];
+#pragma unroll
+            for (int i = 0; i < kLaneTerms; ++i) x[i] = S.term_at(off[i]);
+        });
     };
     for (int step = 0; step < chunk; ++step) {
         const uint32_t gstep = step0 + (uint32_t)step;
@@ -365,14 +458,24 @@ __device__ __forceinline__ void run_steps(const SlotDesc &d, State &S, BatchWall
             // CTA's ends takes the general (EDGE) path for all its rows, so
             // the collision is never executed twice by a diverged warp
             const bool edge = __any_sync(__activemask(), j < j0 + 3 || j >= j1 - 3);
-            if (edge) cell_update<Q, true, PRECISE>(d, S, j, sw, gstep);
-            else cell_update<Q, false, PRECISE>(d, S, j, sw, gstep);
+            cell_update<Q, PRECISE>(d, S, j, edge, sw, gstep);
         }
         const bool more = step + 1 < chunk;
         if (CL == 1) {
-            __syncthreads();
-            S.flip();
-            if (wall_warp && more) fill_next(gstep + 1u);
+            if constexpr (State::kTwoBuffers) {
+                // while the other warps run ahead: the wall warps' rows then
+                // have their SM sub-partitions to themselves
+                __syncthreads();
+                S.flip();
+                if (wall_warp && more) fill_next(gstep + 1u);
+            } else {
+                // before the barrier: afterwards another warp may store to the
+                // slots (of a ring) of what has left the column
+                __syncwarp();
+                S.flip();
+                if (wall_warp && more) fill_next(gstep + 1u);
+                __syncthreads();
+            }
         } else {
             // the next step's wall sums read only rows this warp has just
             // written (visible to it after __syncwarp), so they run between
@@ -385,19 +488,25 @@ __device__ __forceinline__ void run_steps(const SlotDesc &d, State &S, BatchWall
     }
 }
 
-// Up to d.sub chunks of one slot on CTA `rank` of its CL-CTA cluster
-// (fewer when the slot stops: converged, stagnated, non-finite or at
-// max_steps); returns the chunks run.  chunks0 / steps0 are the slot's
+// The chunks of one launch for one slot on CTA `rank` of its CL-CTA cluster:
+// d.sub of them, and then more while another one, as long as those so far,
+// ends before `budget` ns from t0 - the time the slowest slot of the last launch
+// took, for which this launch lasts anyway (fewer when the slot stops:
+// converged, stagnated, non-finite or at max_steps); returns the chunks run.
+// Results do not depend on how many chunks a launch runs: 128 mixed columns on
+// 304 CTAs, whose tall one-CTA columns take 2.3 ms per chunk and clusters 0.2 -
+// 0.7, 473 -> 414 ms to the last one's steady state.  chunks0 / steps0 are the slot's
 // counters before the launch (read by every CTA before the first barrier);
 // `part` the slot's per-chunk FP64 partial sums of the residual; `sm` the
-// CTA's kSmemBytes of dynamic shared memory (used when R <= kSmemRows).  A
+// CTA's kSmemBytes of dynamic shared memory (used when its rows fit).  A
 // residual check follows every check_every-th chunk of the slot's count, so
 // the checks fall on the same steps whatever the number of chunks per launch.
 template <int Q>
 __device__ __forceinline__ int batch_slot(const SlotDesc &d, float *__restrict__ pool,
                                           SlotStatus *__restrict__ st, BatchWallShared &sw,
                                           int rank, int CL, int chunks0, long long steps0,
-                                          int precise, double *__restrict__ part, float *sm) {
+                                          int precise, double *__restrict__ part, float *sm,
+                                          unsigned long long t0, unsigned long long budget) {
     using L = Lat<Q>;
     const int chunk = d.chunk_steps;
     const KConsts<float> &k = d.k;
@@ -420,10 +529,10 @@ __device__ __forceinline__ int batch_slot(const SlotDesc &d, float *__restrict__
         nt = min(32, span);
     }
     const int mb = j0 + nb, me = j1 - nt;
-    const bool smem = batch_uses_smem(Ny, CL);
+    const bool smem = batch_uses_smem(Ny, CL, k.accom[0] == 1.0 && k.accom[1] == 1.0);
 
     // Change of the macroscopic fields since the last check (Eq. (3) moments
-    // of the state `fin` after chunk ck), in the units of the accuracy the
+    // of the state after chunk ck, read through at(a, e_y, local row)), in the units of the accuracy the
     // solve is asked for: over the 32-row blocks of the column, the largest
     // change of a block's mean u_x divided by the wall speed u_ref, and for a
     // thermal lattice also the largest change of a block's mean T.  The block
@@ -434,7 +543,7 @@ __device__ __forceinline__ int batch_slot(const SlotDesc &d, float *__restrict__
     // the blocks in a fixed order: the result does not depend on how the rows
     // were split across CTAs.  Returns whether the slot keeps running (the
     // same answer in every thread of the cluster).
-    auto check = [&](const float *fin, int ck, long long steps_k) -> bool {
+    auto check = [&](auto &&at, int ck, long long steps_k) -> bool {
         float *prev_u = (float *)(pool + d.prev_off);
         float *prev_T = prev_u + Ny;
         const double r = (double)k.r;
@@ -447,8 +556,8 @@ __device__ __forceinline__ int batch_slot(const SlotDesc &d, float *__restrict__
                 double s0 = 0, sx = 0, sy = 0, se = (double)k.e2w;
 #pragma unroll
                 for (int a = 0; a < Q; ++a) {
-                    const double fa = smem ? (double)fin[(j - j0) * Q + a]
-                                           : (double)__ldcg(fin + (long long)a * Ny + j);
+                    const float *p = at(a, L::ey(a), j - j0);
+                    const double fa = smem ? (double)*p : (double)__ldcg(p);
                     s0 += fa;
                     sx += L::ex(a) * fa;
                     sy += L::ey(a) * fa;
@@ -546,11 +655,10 @@ __device__ __forceinline__ int batch_slot(const SlotDesc &d, float *__restrict__
             // systematic round-off: restore the admission mass, spread over
             // the cells as rest equilibrium (d_a += dm w_a, no momentum)
             const float dm = (float)((d.mass0 - __ldcg(&st->mass)) / (double)Ny);
-            float *f = const_cast<float *>(fin);
             for (int j = j0 + tid; j < j1; j += nth)
 #pragma unroll
                 for (int a = 0; a < Q; ++a) {
-                    float &v = smem ? f[(j - j0) * Q + a] : f[(long long)a * Ny + j];
+                    float &v = *at(a, L::ey(a), j - j0);
                     v = __fmaf_rn(dm, k.w[a], v);
                 }
             slot_barrier(CL);                  // every CTA read precise == 2 and corrected
@@ -561,10 +669,10 @@ __device__ __forceinline__ int batch_slot(const SlotDesc &d, float *__restrict__
     };
     // after sub-chunk kk of this launch: a check when the slot's chunk count
     // calls for one, else the counters (and the max_steps stop)
-    auto after_chunk = [&](const float *fin, int kk) -> bool {
+    auto after_chunk = [&](auto &&at, int kk) -> bool {
         const int ck = chunks0 + kk;
         const long long steps_k = steps0 + (long long)kk * chunk;
-        if (ck % d.check_every == 0) return check(fin, ck, steps_k);
+        if (ck % d.check_every == 0) return check(at, ck, steps_k);
         if (rank == 0 && tid == 0) {
             st->chunks = ck;
             st->steps = steps_k;
@@ -573,43 +681,71 @@ __device__ __forceinline__ int batch_slot(const SlotDesc &d, float *__restrict__
         return steps_k < d.max_steps;
     };
 
+    // one more chunk in this launch?  (the same answer in every thread of the cluster)
+    auto another = [&](int done) -> bool {
+        if (done < d.sub) return true;
+        if (rank == 0 && tid == 0) {
+            const unsigned long long el = global_ns() - t0;
+            if (done == d.sub) st->first_ns = (long long)el;
+            st->go = done < kMaxLaunchChunks && el + el / (unsigned)done <= budget;
+        }
+        slot_barrier(CL);
+        return __ldcg(&st->go) != 0;
+    };
+
     float *g_cur = pool + d.f_off + (d.cur ? (long long)Q * Ny : 0);
     float *g_oth = pool + d.f_off + (d.cur ? 0 : (long long)Q * Ny);
     if (tid < 2) sw.acc[tid] = (float)k.accom[tid];
     int done = 0;
-    if (smem) {
-        // own rows into buffer 0, transposed to rows of Q populations
+    auto run_smem = [&](auto ring) {
+        constexpr bool RING = decltype(ring)::value;
+        // own rows into slots 0, 1, ... (t = 0)
         for (int i = tid; i < Q * span; i += nth) {
             const int a = i / span, r = i - a * span;
             sm[r * Q + a] = __ldcg(g_cur + (long long)a * Ny + j0 + r);
         }
         const uint32_t base = (uint32_t)__cvta_generic_to_shared(sm);
-        SmemState<Q> S{base, 0u, 0u, map_rank(base, rank), R, j0, 0};
+        SmemState<Q, RING> S{base, 0u, 0u, map_rank(base, rank), R, j0, Ny, 0};
         if (rank > 0) S.lo = map_rank(base, rank - 1);
         if (rank < CL - 1) S.hi = map_rank(base, rank + 1);
         slot_barrier(CL);                      // every CTA loaded before any neighbour reads
-        while (done < d.sub) {
+        for (;;) {
             const uint32_t s0 = (uint32_t)(steps0 + (long long)done * chunk);
             if (precise) run_steps<Q, true>(d, S, sw, chunk, CL, warp, lane, tid, nth, j0, j1, nb, nt, mb, me, s0);
             else run_steps<Q, false>(d, S, sw, chunk, CL, warp, lane, tid, nth, j0, j1, nb, nt, mb, me, s0);
             ++done;
-            if (!after_chunk(sm + S.b * Q * R, done)) break;
+            // element of population a (vertical component e) of local row r
+            const int t = S.t;
+            auto at = [=](int a, int e, int r) -> float * {
+                const int sl = RING ? (r - e * t) & (kRing - 1) : t * (kRing / 2) + r;
+                return sm + sl * Q + a;
+            };
+            if (!after_chunk(at, done) || !another(done)) break;
         }
         // write the final state back to the pool buffer it came from
-        const float *fin = sm + S.b * Q * R;
-        for (int i = tid; i < Q * span; i += nth) {
-            const int a = i / span, r = i - a * span;
-            g_cur[(long long)a * Ny + j0 + r] = fin[r * Q + a];
-        }
+        StaticFor<0, Q>::run([&](auto ic) {
+            constexpr int a = decltype(ic)::value;
+            for (int r = tid; r < span; r += nth)
+                g_cur[(long long)a * Ny + j0 + r] = sm[S.slot_of(r, L::ey(a)) * Q + a];
+        });
+    };
+    if (smem && R <= kRing / 2) {
+        run_smem(std::false_type{});
+    } else if (smem) {
+        run_smem(std::true_type{});
     } else {
         __syncthreads();
         GlobalState S{g_cur, g_oth, Ny, &sw.term[0][0][0]};
-        while (done < d.sub) {
+        for (;;) {
             const uint32_t s0 = (uint32_t)(steps0 + (long long)done * chunk);
             if (precise) run_steps<Q, true>(d, S, sw, chunk, CL, warp, lane, tid, nth, j0, j1, nb, nt, mb, me, s0);
             else run_steps<Q, false>(d, S, sw, chunk, CL, warp, lane, tid, nth, j0, j1, nb, nt, mb, me, s0);
             ++done;
-            if (!after_chunk(S.src, done)) break;
+            const float *src = S.src;
+            auto at = [=](int a, int, int r) -> float * {
+                return const_cast<float *>(src) + (long long)a * Ny + j0 + r;
+            };
+            if (!after_chunk(at, done) || !another(done)) break;
         }
     }
     return done;

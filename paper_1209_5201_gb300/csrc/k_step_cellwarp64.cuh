@@ -25,7 +25,6 @@
 
 #include <type_traits>
 
-#include "k_step_staged.cuh"                // global_ns
 #include "lbm_device.cuh"
 
 namespace lbm {
@@ -263,7 +262,7 @@ k_steps_cellwarp64_cluster(const double *fin, double *fout,
     const bool live = cell < k.Nx * k.Ny;
     double *sf = s_f[warp];
     if (lane < QP - Q) sf[Q + lane] = 0.0;
-    const uint32_t base = smem_addr(&s_st[0][0][0]);
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(&s_st[0][0][0]);
     constexpr uint32_t kBuf = kCellWarps * QP * 8u;
     Lane cl;
     double va = 0.0, vb = 0.0;

@@ -53,11 +53,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
 // bounded wait: false when limit_ns ran out; a zero limit gives up at once,
 // whether or not the phase has completed (the failure path, on demand)
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity,

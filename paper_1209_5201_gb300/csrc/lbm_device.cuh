@@ -48,6 +48,12 @@ LBM_DEFINE_LAT(17, 5, LBM_Q17_EX, LBM_Q17_EY, LBM_Q17_SH)
 LBM_DEFINE_LAT(25, 6, LBM_Q25_EX, LBM_Q25_EY, LBM_Q25_SH)
 LBM_DEFINE_LAT(37, 8, LBM_Q37_EX, LBM_Q37_EY, LBM_Q37_SH)
 
+__device__ __forceinline__ unsigned long long global_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
 // ---- storage formats ---------------------------------------------------------
 template <int PREC> struct Store;
 // dev:     stored d_a = f~*_a - w_a rho with rho the cell's own density,

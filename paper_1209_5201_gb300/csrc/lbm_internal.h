@@ -124,6 +124,16 @@ struct KWall {
     signed char out_a[2][kMaxWallOut];
 };
 
+// c0 + d c with both constants split into pairs of floats.
+inline KWall::Emit wall_emit(double c, double c0) {
+    KWall::Emit e;
+    e.ch = (float)c;
+    e.cl = (float)(c - (double)e.ch);
+    e.c0h = (float)c0;
+    e.c0l = (float)(c0 - (double)e.c0h);
+    return e;
+}
+
 // Constants of the FP64 one-warp-per-cell step by lane (k_step_cellwarp64.cuh):
 // lane 0 the rest velocity, lane p the pair (2p - 1, 2p), whose first member's
 // velocity is (ex, ey).

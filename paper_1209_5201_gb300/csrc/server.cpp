@@ -104,6 +104,9 @@ struct ServerImpl {
     long long *d_off = nullptr;
     int *d_dbg = nullptr;                    // kernels' record of a rejected descriptor
     int *h_dbg = nullptr;
+    // time of the slowest running slot's part of the last launch: the others
+    // run further chunks within it
+    unsigned long long *d_budget = nullptr, *h_budget = nullptr;
     double *d_out = nullptr;                 // read-out staging
     long long out_elems = 0;
     // host mirrors (pinned)
@@ -255,27 +258,30 @@ struct ServerImpl {
         // e.n < -l); the bottom list takes e_y < 0 at rows 0..|e_y|-1, the top
         // list e_y > 0 at rows Ny-1.. (distance from the wall)
         int nb = 0, nt = 0;
-        for (int a = 0; a < L.Q; ++a) {
-            for (int kk = 0; kk < -L.ey[a]; ++kk) { d.term_a[0][nb] = (signed char)a; d.term_row[0][nb] = (signed char)kk; ++nb; }
-            for (int kk = 0; kk < L.ey[a]; ++kk) { d.term_a[1][nt] = (signed char)a; d.term_row[1][nt] = (signed char)kk; ++nt; }
-        }
-        if (nb != nt || nb >= 32) std::abort();  // lattices are symmetric, <= 26 terms
+        for (int a = 0; a < L.Q; ++a)
+            for (int kk = 0; kk < std::abs(L.ey[a]); ++kk) {
+                const int w = L.ey[a] < 0 ? 0 : 1, l = w == 0 ? nb++ : nt++;
+                d.term_a[w][l] = (signed char)a;
+                d.term_row[w][l] = (signed char)kk;
+                d.term_ey[w][l] = (signed char)L.ey[a];
+            }
+        if (nb != nt || nb > kMaxTerm) std::abort();  // lattices are symmetric, <= 26 terms
         d.nterm = nb;
         fill_consts(d.k, L, p, 1);
-        // the wall warp sums the terms' deviations d = f - w and adds their
-        // weights once (wterm); it then forms M_in g^w_a / D_w - w_a for the
-        // outgoing velocities of its wall (e_y > 0 bottom, e_y < 0 top)
+        // the wall warp sums the terms' deviations d = f - w and forms
+        // M_in g^w_a / D_w - w_a of the outgoing velocities of its wall (e_y > 0
+        // bottom, e_y < 0 top), the terms' weights in the constants
+        double wterm[2] = {0.0, 0.0};
+        for (int a = 0; a < L.Q; ++a)
+            for (int kk = 0; kk < std::abs(L.ey[a]); ++kk) wterm[L.ey[a] < 0 ? 0 : 1] += (double)d.k.w[a];
         int no[2] = {0, 0};
         for (int a = 0; a < L.Q; ++a) {
-            for (int kk = 0; kk < -L.ey[a]; ++kk) d.wterm[0] += (double)d.k.w[a];
-            for (int kk = 0; kk < L.ey[a]; ++kk) d.wterm[1] += (double)d.k.w[a];
             const int wl = L.ey[a] > 0 ? 0 : (L.ey[a] < 0 ? 1 : -1);
             if (wl < 0) continue;
-            if (no[wl] >= kMaxOut || !(d.k.wcoef[wl][a] > 0.0)) std::abort();
+            const double c = d.k.wcoef[wl][a];
+            if (no[wl] >= kMaxOut || !(c > 0.0)) std::abort();
             d.out_a[wl][no[wl]] = (signed char)a;
-            d.out_c[wl][no[wl]] = d.k.wcoef[wl][a];
-            d.out_w[wl][no[wl]] = (double)d.k.w[a];
-            ++no[wl];
+            d.out_e[wl][no[wl]++] = wall_emit(c, std::fma(wterm[wl], c, -(double)d.k.w[a]));
         }
         if (no[0] != no[1] || no[0] < 1) std::abort();
         d.nout = no[0];
@@ -365,13 +371,14 @@ struct ServerImpl {
     // and a join on `st`, so that the classes run concurrently (also inside
     // the captured graph).
     cudaError_t launch_chunks(cudaStream_t st) {
-        cudaError_t e = cudaEventRecord(ev_fork, st);
+        cudaError_t e = cudaMemcpyAsync(d_budget, h_budget, sizeof(*h_budget), cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaEventRecord(ev_fork, st);
         for (int c = 0; c < kBatchClasses && e == cudaSuccess; ++c) {
             e = cudaStreamWaitEvent(side[c], ev_fork, 0);
             if (e == cudaSuccess)
                 e = (cudaError_t)launch_batch_chunk(side[c], d_desc, d_status, pool, d_part,
                                                     cls_base[c], cls_cap[c], kBatchClassCL[c],
-                                                    pool_elems, d_dbg);
+                                                    pool_elems, d_budget, d_dbg);
             if (e == cudaSuccess) e = cudaEventRecord(ev_join[c], side[c]);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev_join[c], 0);
         }
@@ -575,6 +582,15 @@ struct ServerImpl {
         nvtxRangePop();
         if (e) return fail("chunk", e);
         if (h_dbg[0]) return reject_desc();
+        // (a launch with requests still waiting for the next one keeps to its
+        // slowest slot's chunks)
+        {
+            std::unique_lock<std::mutex> lk(mu);
+            *h_budget = queue.empty() && admitted.empty() ? kMinLaunchNs : 0;
+        }
+        for (int s = 0; s < (int)slots.size(); ++s)
+            if (slots[s].busy && h_status[s].state == kSlotRunning)
+                *h_budget = std::max(*h_budget, (unsigned long long)h_status[s].first_ns);
         ++chunks;
         occupancy_sum += used_ctas;
         // retire finished slots
@@ -791,6 +807,8 @@ int lbm_server_create(const lbm_server_cfg *cfg, void *stream, lbm_server **out)
         ck(cudaMallocAsync((void **)&S.d_out, sizeof(double) * S.out_elems, S.stream));
         ck(cudaMallocAsync((void **)&S.d_dbg, sizeof(int) * 8, S.stream));
         ck(cudaMallocHost((void **)&S.h_dbg, sizeof(int) * 8));
+        ck(cudaMallocAsync((void **)&S.d_budget, sizeof(*S.d_budget), S.stream));
+        ck(cudaMallocHost((void **)&S.h_budget, sizeof(*S.h_budget)));
         ck(cudaMallocHost((void **)&S.h_desc, sizeof(SlotDesc) * ns));
         ck(cudaMallocHost((void **)&S.h_status, sizeof(SlotStatus) * ns));
         ck(cudaMallocHost((void **)&S.h_idx, sizeof(int) * ns));
@@ -803,6 +821,7 @@ int lbm_server_create(const lbm_server_cfg *cfg, void *stream, lbm_server **out)
             ck(cudaMemcpyAsync(S.d_status, S.h_status, sizeof(SlotStatus) * ns, cudaMemcpyHostToDevice, S.stream));
             ck(cudaMemsetAsync(S.d_dbg, 0, sizeof(int) * 8, S.stream));
             std::memset(S.h_dbg, 0, sizeof(int) * 8);
+            *S.h_budget = kMinLaunchNs;
             ck(cudaStreamSynchronize(S.stream));
         }
         if (e == cudaSuccess && cfg->use_graph) {
@@ -977,6 +996,7 @@ int lbm_server_destroy(lbm_server *h) {
     if (S.d_idx) cudaFreeAsync(S.d_idx, S.stream);
     if (S.d_off) cudaFreeAsync(S.d_off, S.stream);
     if (S.d_out) cudaFreeAsync(S.d_out, S.stream);
+    if (S.d_budget) cudaFreeAsync(S.d_budget, S.stream);
     if (S.d_dbg) cudaFreeAsync(S.d_dbg, S.stream);
     if (S.d_part) cudaFreeAsync(S.d_part, S.stream);
     cudaStreamSynchronize(S.stream);
@@ -991,6 +1011,7 @@ int lbm_server_destroy(lbm_server *h) {
     if (S.h_off) cudaFreeHost(S.h_off);
     if (S.h_out) cudaFreeHost(S.h_out);
     if (S.h_dbg) cudaFreeHost(S.h_dbg);
+    if (S.h_budget) cudaFreeHost(S.h_budget);
     delete h;
     return LBM_OK;
 }
