@@ -41,9 +41,16 @@
 namespace lbm {
 namespace {
 
-// work above which a request counts as long for the cluster choice: row-steps
-// per thread on one CTA (~1 s at ~4 us per step and 256 rows)
-constexpr double kLongRowSteps = 2.5e5;
+// work above which a request gets a cluster, row-steps per thread on one CTA: at
+// admission, when more requests may be about to arrive (~1 s at ~4 us per step
+// and 256 rows), and while running, once CTAs are spare (about 50 ms; at 2.5e5
+// the last 200 ms of 128 mixed solves ran on one CTA per column with most of
+// the GPU idle, and at 2e4 on admission the first requests of a burst took the
+// CTAs of its last ones).
+constexpr double kLongRowSteps = 2.5e5, kGrowRowSteps = 2e4;
+// rows per CTA that fit its shared memory however the column is split (whole
+// 32-row residual chunks, three slots of the 512 free)
+constexpr int kFitRows = 480;
 constexpr long long kAlignElems = 64;        // 256-byte granularity (floats)
 // A request's collision rounds to nearest while its change per check is above
 // kPreciseFrom x tol (far from the steady state the state changes every step,
@@ -306,11 +313,11 @@ struct ServerImpl {
         si.elems = request_elems(r, L.Q);
     }
 
-    cudaError_t upload_slot(int s) {
-        cudaError_t e = cudaMemcpyAsync(d_desc + s, h_desc + s, sizeof(SlotDesc),
+    cudaError_t upload_slots(int s, int n) {
+        cudaError_t e = cudaMemcpyAsync(d_desc + s, h_desc + s, n * sizeof(SlotDesc),
                                         cudaMemcpyHostToDevice, stream);
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(d_status + s, h_status + s, sizeof(SlotStatus),
+            e = cudaMemcpyAsync(d_status + s, h_status + s, n * sizeof(SlotStatus),
                                 cudaMemcpyHostToDevice, stream);
         return e;
     }
@@ -337,7 +344,7 @@ struct ServerImpl {
     // one CTA (a barrier per step across the cluster), so it is only worth its
     // latency gain for long requests: estimated row-steps per thread on one
     // CTA (14 e-folding times of the slowest shear mode, Ny / 256 rows per
-    // thread) above kLongRowSteps.  Results do not depend on the split: every
+    // thread) of `least` at least.  Results do not depend on the split: every
     // cell update is the same arithmetic on the same values, chunk lengths and
     // checks ignore the cluster, and the residual is summed over 32-row chunks
     // in a fixed order.
@@ -351,11 +358,19 @@ struct ServerImpl {
                                        : 0.127 * r.Ny * L.r / r.Kn + 1.2 * r.Ny * L.r;
         return 14.0 * efold;
     }
-    bool long_split(const lbm_request &r, int &cl, double &work) const {
+    bool long_split(const lbm_request &r, int &cl, double &work, double least) const {
         cl = batch_cluster_size(r.Ny, cfg.cluster_rows, cfg.max_slots, max_cl);
         if (cl == 1) return false;
-        work = est_steps(r) * std::ceil(r.Ny / 256.0);
-        return work >= kLongRowSteps;
+        work = std::min(est_steps(r), (double)r.max_steps) * std::ceil(r.Ny / 256.0);
+        return work >= least;
+    }
+
+    // the cluster whose CTAs hold a column's rows in shared memory (1 where a
+    // configured cluster_rows beyond that keeps it whole)
+    int fit_cluster(const lbm_request &r) const {
+        const bool diffuse = r.accom[0] == 1.0 && r.accom[1] == 1.0;
+        if (r.Ny <= (diffuse ? 512 : 509)) return 1;
+        return batch_cluster_size(r.Ny, std::max(kFitRows, (int)cfg.cluster_rows), cfg.max_slots, max_cl);
     }
 
     // a free slot of the class of clusters of cl CTAs, or -1
@@ -397,10 +412,11 @@ struct ServerImpl {
     // CTA on a full GPU) and set the latency tail.
     double remaining(int s) const {
         // remaining row-steps on one CTA; a request past its estimate keeps a
-        // quarter of it
-        const double est = est_steps(slots[s].req);
-        return std::max(est - (double)h_status[s].steps, 0.25 * est) *
-               std::ceil(slots[s].req.Ny / 256.0);
+        // quarter of it, none more than its step limit leaves
+        const lbm_request &r = slots[s].req;
+        const double est = est_steps(r), done = (double)h_status[s].steps;
+        return std::min(std::max(est - done, 0.25 * est), (double)r.max_steps - done) *
+               std::ceil(r.Ny / 256.0);
     }
     cudaError_t rebalance(long long spare, int short_ctas, const std::vector<int> &fresh) {
         struct Cand { double rem; int s; };
@@ -434,9 +450,9 @@ struct ServerImpl {
                 if (!movable(s)) continue;
                 int cl;
                 double work;
-                if (!long_split(slots[s].req, cl, work) || cl <= h_desc[s].cl) continue;
+                if (!long_split(slots[s].req, cl, work, kGrowRowSteps) || cl <= h_desc[s].cl) continue;
                 const double rem = remaining(s);
-                if (rem >= kLongRowSteps) cand.push_back({rem, s});
+                if (rem >= kGrowRowSteps) cand.push_back({rem, s});
             }
             std::sort(cand.begin(), cand.end(), [](const Cand &x, const Cand &y) { return x.rem > y.rem; });
             for (const Cand &c : cand) {
@@ -476,8 +492,8 @@ struct ServerImpl {
             h_status[m.from].state = kSlotIdle;
             if (m.cl > from_cl) ++promoted;
             else ++demoted;
-            if (e == cudaSuccess) e = upload_slot(m.to);
-            if (e == cudaSuccess) e = upload_slot(m.from);
+            if (e == cudaSuccess) e = upload_slots(m.to, 1);
+            if (e == cudaSuccess) e = upload_slots(m.from, 1);
         }
         return e;
     }
@@ -498,35 +514,46 @@ struct ServerImpl {
                         stopped.push_back(s);
                     }
             cancels.clear();
-            // CTAs beyond one for every queued request go to the longest queued
-            // requests (among the first 512), longest first, as clusters: the
+            // CTAs beyond one for every queued request go to queued requests
+            // (among the first 512) as clusters: the
             // GPU's idle CTAs shorten the requests that set the latency tail,
             // and none is taken from a request still waiting.
             std::map<uint64_t, int> split;
             long long extra = (long long)cfg.max_slots - used_ctas - (long long)queue.size();
             if (extra > 0) {
-                std::vector<std::pair<double, std::pair<uint64_t, int>>> cand;
+                std::vector<std::pair<double, std::pair<uint64_t, int>>> fit, cand;
                 int n = 0;
                 for (auto q = queue.begin(); q != queue.end() && n < 512; ++q, ++n) {
-                    int cl;
+                    int cl = fit_cluster(q->req);
+                    if (cl > 1) fit.push_back({(double)q->req.Ny * lattice_q(q->req.lattice), {q->id, cl}});
                     double work;
-                    if (long_split(q->req, cl, work)) cand.push_back({work, {q->id, cl}});
+                    if (long_split(q->req, cl, work, kLongRowSteps)) cand.push_back({work, {q->id, cl}});
                 }
-                std::sort(cand.begin(), cand.end(),
-                          [](const auto &x, const auto &y) { return x.first > y.first; });
-                for (const auto &c : cand)
-                    if (extra >= c.second.second - 1) {
-                        split[c.second.first] = c.second.second;
-                        extra -= c.second.second - 1;
+                // first the columns whose rows one CTA's shared memory does not
+                // hold, tallest first: from L2 a CTA advances 65 rows per us on
+                // a full GPU, from shared memory 110, and the tallest set a
+                // launch's length; then longest first
+                const auto down = [](const auto &x, const auto &y) { return x.first > y.first; };
+                std::stable_sort(fit.begin(), fit.end(), down);
+                std::stable_sort(cand.begin(), cand.end(), down);
+                for (const auto *list : {&fit, &cand})
+                    for (const auto &c : *list) {
+                        int &have = split.emplace(c.second.first, 1).first->second;
+                        if (c.second.second > have && extra >= c.second.second - have) {
+                            extra -= c.second.second - have;
+                            have = c.second.second;
+                        }
                     }
             }
-            // Scan the queue in arrival order (at most 64 entries).  A request
+            // Scan the queue in arrival order (at most 1024 entries: a burst is
+            // admitted at once, for every launch that it is spread over is one
+            // that its last requests wait for).  A request
             // is admitted when its class has a free slot and its cluster fits
             // the CTA budget (max_slots) minus what the oldest request that did
             // not fit needs (so that later requests cannot starve it); the
             // first request that finds no memory stops the scan.
             int reserve = 0, scanned = 0;
-            for (auto it = queue.begin(); it != queue.end() && scanned < 64; ++scanned) {
+            for (auto it = queue.begin(); it != queue.end() && scanned < 1024; ++scanned) {
                 const auto sp = split.find(it->id);
                 const int cl = sp == split.end() ? 1 : sp->second;
                 const bool fits = used_ctas + cl + reserve <= cfg.max_slots;
@@ -557,9 +584,13 @@ struct ServerImpl {
         if (idle) return LBM_OK;
         if ((e = rebalance(spare, short_ctas, admitted))) return fail("rebalance", e);
         if (!admitted.empty()) {
-            // only the admitted entries: running slots' buffer index lives on the device
-            for (int s : admitted)
-                if ((e = upload_slot(s))) return fail("upload slot", e);
+            // only the admitted entries (running slots' buffer index lives on the
+            // device), neighbouring slots in one copy
+            std::sort(admitted.begin(), admitted.end());
+            for (size_t i = 0, n; i < admitted.size(); i += n) {
+                for (n = 1; i + n < admitted.size() && admitted[i + n] == admitted[i] + (int)n;) ++n;
+                if ((e = upload_slots(admitted[i], (int)n))) return fail("upload slot", e);
+            }
             for (size_t i = 0; i < admitted.size(); ++i) h_idx[i] = admitted[i];
             if ((e = cudaMemcpyAsync(d_idx, h_idx, sizeof(int) * admitted.size(), cudaMemcpyHostToDevice, stream)))
                 return fail("upload slot list", e);
@@ -660,8 +691,10 @@ struct ServerImpl {
         }
         if (!fin.empty()) {
             // idle the retired slots on the device too
-            for (int s : fin)
-                if ((e = upload_slot(s))) return fail("upload slot", e);
+            for (size_t i = 0, n; i < fin.size(); i += n) {
+                for (n = 1; i + n < fin.size() && fin[i + n] == fin[i] + (int)n;) ++n;
+                if ((e = upload_slots(fin[i], (int)n))) return fail("upload slot", e);
+            }
             cv_done.notify_all();
         }
         return LBM_OK;
