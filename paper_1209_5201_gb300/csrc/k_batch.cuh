@@ -440,6 +440,15 @@ __device__ __forceinline__ void run_steps(const SlotDesc &d, State &S, BatchWall
             }
         });
     }
+    // A full ring (510 to 512 rows on one CTA) has no slot between what leaves
+    // the column and what enters it.  Step t moves velocity e of row lr into slot
+    // (lr - (t + 1) e) mod 512, where before it stood row lr - e; for lr - e < 0
+    // or >= 512 that is row lr - e + 512 or - 512, one of the terms just read
+    // (512 rows, e = 1: row 0 stores where row 511's term is; 510 rows, e = 3:
+    // row 0 where row 509's is; 509 rows: no such row).  So every wall sum has
+    // read its terms before any warp stores: here for the chunk's first step,
+    // before the step's barrier for the others.
+    if (!State::kTwoBuffers && CL == 1) __syncthreads();
     auto fill_next = [&](uint32_t st) {
         wall_fill_warp(d, wall, lane, sw.fill[wall], st, [&](const int (&t)[kLaneTerms], float (&x)[kLaneTerms]) {
             int off[kLaneTerms];
