@@ -25,8 +25,8 @@ __device__ __forceinline__ C warp_allsum(C v) {
 
 template <int Q, int PREC>
 __global__ void __launch_bounds__(32)
-k_step_cellwarp(const typename Store<PREC>::S *__restrict__ fin,
-                typename Store<PREC>::S *__restrict__ fout, const float *__restrict__ rin,
+k_step_cellwarp(const typename Store<PREC>::S *fin,
+                typename Store<PREC>::S *__restrict__ fout, const float *rin,
                 float *__restrict__ rout,
                 const __grid_constant__ KConsts<typename Store<PREC>::C> k,
                 const __grid_constant__ KWall kw) {
@@ -58,6 +58,8 @@ k_step_cellwarp(const typename Store<PREC>::S *__restrict__ fin,
     // launched with programmatic stream serialization: the previous step may
     // still be running; let the next step's launch begin, then wait for the
     // previous grid to complete (its stores visible) before touching the state
+    // (fin and rin, which it writes, are not __restrict__: that would let loads
+    // move above the wait)
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const int j = blockIdx.x / k.Nx, x = blockIdx.x - j * k.Nx;

@@ -27,8 +27,8 @@ namespace lbm {
 template <int PREC, int BX>
 using WallFills = typename Store<PREC>::C[kMaxWallOut][BX + 6];
 template <int Q, int PREC, int BX>
-__device__ __forceinline__ void wall_prologue(const typename Store<PREC>::S *__restrict__ fin,
-                                              const float *__restrict__ rin,
+__device__ __forceinline__ void wall_prologue(const typename Store<PREC>::S *fin,
+                                              const float *rin,
                                               const KConsts<typename Store<PREC>::C> &k,
                                               const KWall &kw, int wall, int x0, int ncols,
                                               WallFills<PREC, BX> &s_fill) {
@@ -40,10 +40,10 @@ __device__ __forceinline__ void wall_prologue(const typename Store<PREC>::S *__r
 // tile, rsrc its density (BF16DEV).  PC > 0: the tile pitch, a compile-time
 // constant; PC = 0: the solver's pitch, offsets from the constants.
 template <int Q, int PREC, int BX, bool WALL, int PC>
-__device__ __forceinline__ void pull(const typename Store<PREC>::S *__restrict__ fin,
-                                     const float *__restrict__ rin,
-                                     const typename Store<PREC>::S *__restrict__ src,
-                                     const float *__restrict__ rsrc,
+__device__ __forceinline__ void pull(const typename Store<PREC>::S *fin,
+                                     const float *rin,
+                                     const typename Store<PREC>::S *src,
+                                     const float *rsrc,
                                      const KConsts<typename Store<PREC>::C> &k, const KWall &kw,
                                      int x, int j, const WallFills<PREC, BX> &s_fill,
                                      typename Store<PREC>::C (&f)[Q]) {
@@ -214,8 +214,8 @@ __device__ __forceinline__ void collide_store(const typename Store<PREC>::C (&f)
 // = tile * ceil(tw / BX) + block of the tile.
 template <int Q, int PREC, int BX, int MINB, bool CS, int RS, int PC, bool ISO2>
 __global__ void __launch_bounds__(BX, MINB)
-k_step_direct(const typename Store<PREC>::S *__restrict__ fin,
-              typename Store<PREC>::S *__restrict__ fout, const float *__restrict__ rin,
+k_step_direct(const typename Store<PREC>::S *fin,
+              typename Store<PREC>::S *__restrict__ fout, const float *rin,
               float *__restrict__ rout,
               const __grid_constant__ KConsts<typename Store<PREC>::C> k,
               const __grid_constant__ KWall kw) {
@@ -236,7 +236,8 @@ k_step_direct(const typename Store<PREC>::S *__restrict__ fin,
     const int j1 = min(k.Ny, j0 + RS);
     const bool bot = j0 < L::N, top = j1 > k.Ny - L::N;
     const int ncols = min(BX, w - xl0) + 6;
-    // the previous step's stores are visible from here on
+    // the previous step's stores are visible from here on (fin and rin, which it
+    // writes, are not __restrict__: that would let loads move above the wait)
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     if (RS > 1) {
         if (bot) wall_prologue<Q, PREC, BX>(fin, rin, k, kw, 0, t * k.tw + xl0, ncols, s_fill[0]);

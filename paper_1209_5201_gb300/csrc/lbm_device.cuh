@@ -96,27 +96,30 @@ template <> __device__ __forceinline__ double from_c<double>(double v) { return 
 // ---- addressing of the shifted streams ------------------------------------------
 // A global access at byte offset b (signed) from the 64-bit base p, the
 // offset a per-velocity constant of the solve: the address is one 64-bit add
-// of a warp-uniform constant.  The loads use the read-only path (the source
-// buffer is not written during a step) and ask L2 to fetch the 256-byte
-// block around each 128-byte request: the next warp's shifted segment of the
-// same plane row then hits L2 (about 1 % on the 4096 x 2048 step).
+// of a warp-uniform constant.  The step kernels are launched while the step
+// that writes their source may still run, so the loads are coherent ones
+// (ld.global; the read-only path is for memory that no one writes during the
+// kernel's lifetime) and volatile, which keeps them behind the kernel's wait
+// for that step.  They ask L2 to fetch the 256-byte block around each 128-byte
+// request: the next warp's shifted segment of the same plane row then hits L2
+// (about 1 % on the 4096 x 2048 step).
 template <class S> __device__ __forceinline__ S ld_b(const S *p, long long b);
 template <> __device__ __forceinline__ float ld_b<float>(const float *p, long long b) {
     float v;
-    asm("{\n\t.reg .u64 a;\n\tadd.s64 a, %2, %1;\n\tld.global.nc.L2::256B.f32 %0, [a];\n\t}"
+    asm volatile("{\n\t.reg .u64 a;\n\tadd.s64 a, %2, %1;\n\tld.global.L2::256B.f32 %0, [a];\n\t}"
         : "=f"(v) : "l"(b), "l"(p));
     return v;
 }
 template <> __device__ __forceinline__ double ld_b<double>(const double *p, long long b) {
     double v;
-    asm("{\n\t.reg .u64 a;\n\tadd.s64 a, %2, %1;\n\tld.global.nc.L2::256B.f64 %0, [a];\n\t}"
+    asm volatile("{\n\t.reg .u64 a;\n\tadd.s64 a, %2, %1;\n\tld.global.L2::256B.f64 %0, [a];\n\t}"
         : "=d"(v) : "l"(b), "l"(p));
     return v;
 }
 template <> __device__ __forceinline__ __nv_bfloat16 ld_b<__nv_bfloat16>(const __nv_bfloat16 *p,
                                                                        long long b) {
     unsigned short v;
-    asm("{\n\t.reg .u64 a;\n\tadd.s64 a, %2, %1;\n\tld.global.nc.L2::256B.b16 %0, [a];\n\t}"
+    asm volatile("{\n\t.reg .u64 a;\n\tadd.s64 a, %2, %1;\n\tld.global.L2::256B.b16 %0, [a];\n\t}"
         : "=h"(v) : "l"(b), "l"(p));
     return __ushort_as_bfloat16(v);
 }
@@ -127,21 +130,21 @@ template <class S, long long B> struct LdI;
 template <long long B> struct LdI<float, B> {
     __device__ __forceinline__ static float go(const float *p) {
         float v;
-        asm("ld.global.nc.L2::256B.f32 %0, [%1+%2];" : "=f"(v) : "l"(p), "n"(B));
+        asm volatile("ld.global.L2::256B.f32 %0, [%1+%2];" : "=f"(v) : "l"(p), "n"(B));
         return v;
     }
 };
 template <long long B> struct LdI<double, B> {
     __device__ __forceinline__ static double go(const double *p) {
         double v;
-        asm("ld.global.nc.L2::256B.f64 %0, [%1+%2];" : "=d"(v) : "l"(p), "n"(B));
+        asm volatile("ld.global.L2::256B.f64 %0, [%1+%2];" : "=d"(v) : "l"(p), "n"(B));
         return v;
     }
 };
 template <long long B> struct LdI<__nv_bfloat16, B> {
     __device__ __forceinline__ static __nv_bfloat16 go(const __nv_bfloat16 *p) {
         unsigned short v;
-        asm("ld.global.nc.L2::256B.b16 %0, [%1+%2];" : "=h"(v) : "l"(p), "n"(B));
+        asm volatile("ld.global.L2::256B.b16 %0, [%1+%2];" : "=h"(v) : "l"(p), "n"(B));
         return __ushort_as_bfloat16(v);
     }
 };
@@ -712,7 +715,7 @@ __device__ __noinline__ void wall_fill_exact(float h, float m, float l, const K 
 // when e.n < -l, over all layers).
 template <int Q, int PREC>
 __device__ __forceinline__ void
-wall_column_fill(const typename Store<PREC>::S *__restrict__ fin, const float *__restrict__ rin,
+wall_column_fill(const typename Store<PREC>::S *fin, const float *rin,
                  const KConsts<typename Store<PREC>::C> &k, const KWall &kw, int wall, int xw,
                  typename Store<PREC>::C *out, int stride) {
     using L = Lat<Q>;
@@ -807,7 +810,7 @@ wall_column_fill(const typename Store<PREC>::S *__restrict__ fin, const float *_
 // (Out of line: rare, and inlined per velocity it would double the pull's code.)
 template <int PREC>
 __device__ __noinline__ typename Store<PREC>::C
-specular_source(const typename Store<PREC>::S *__restrict__ fin, const float *__restrict__ rin,
+specular_source(const typename Store<PREC>::S *fin, const float *rin,
                 const KConsts<typename Store<PREC>::C> &k, int a, int ex, int x, int j) {
     const int b = k.mirror[a];
     const int xs = wrap(x - 2 * ex, k.Nx);
