@@ -204,7 +204,7 @@ int lbm_solver_macros(lbm_solver *s, double *rho, double *ux, double *uy,
  * stochastically, so a steady state carries zero-mean noise (about 4e-3 U_w
  * in u_x on the 64-row Couette column) and the mean over a few thousand steps
  * is the steady field to about a tenth of that.  Errors: LBM_EINVAL,
- * LBM_ECUDA, LBM_ETIMEOUT (staged kernel). */
+ * LBM_ECUDA, LBM_ETIMEOUT (a step kernel's bounded wait). */
 int lbm_solver_macros_mean(lbm_solver *s, int64_t nsteps, double *rho, double *ux, double *uy,
                            double *T);
 
@@ -278,13 +278,15 @@ int lbm_solver_set_kernel(lbm_solver *s, int32_t kernel, int32_t variant);
  * library's failure detection.  A wait that runs out records a device flag,
  * the CTA stops taking tiles and its producer waits for its copies in flight
  * (with a fixed 2 s limit of its own) before the CTA exits; the next
- * lbm_solver_sync (or a synchronous call) returns LBM_ETIMEOUT and clears the
- * flag.  The state of that step is then incomplete: reload one (set_state,
- * set_f or init) before stepping on.  0 makes every such wait give up at
- * once, met or not (the failure path on demand; the drain before exit still
- * waits).  FP64 CELLWARP grids advance many steps per launch behind a grid
- * barrier whose waits have a fixed 2 s limit and the same outcome; the other
- * kernels have no waits.  Errors: LBM_EINVAL. */
+ * lbm_solver_sync, lbm_solver_run_to_residual or call that reads the state
+ * out (get_f, get_state, macros, macros_mean, fluxes, wall_mass, stats)
+ * returns LBM_ETIMEOUT and clears the flag.  The state of that step is then
+ * incomplete: reload one (set_state, set_f or init) before stepping on.  0
+ * makes every such wait give up at once, met or not (the failure path on
+ * demand; the drain before exit still waits).  FP64 CELLWARP grids advance
+ * many steps per launch behind a grid barrier whose waits have a fixed 2 s
+ * limit and the same outcome; the other kernels have no waits.
+ * Errors: LBM_EINVAL. */
 int lbm_solver_set_wait_limit(lbm_solver *s, uint64_t ns);
 /* Number of compiled variants of `kernel` (DIRECT or STAGED) for this
  * solver's precision.  Errors: LBM_EINVAL. */

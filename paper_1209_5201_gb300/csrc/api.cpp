@@ -163,12 +163,14 @@ int effective_kernel(const SolverImpl &s) {
     return (long long)s.p.Nx * s.p.Ny <= kCellwarpAutoCells ? LBM_KERNEL_CELLWARP : LBM_KERNEL_DIRECT;
 }
 
-// Error flags the staged kernel raises when a bounded wait runs out.
-int check_device_error(SolverImpl &s) {
-    int flag = 0;
-    CU(cudaMemcpyAsync(&flag, s.derr, sizeof(int), cudaMemcpyDeviceToHost, s.stream));
+// Waits for the stream and reports the flag that a step kernel raises when a
+// bounded wait runs out: the end of every call that hands out the state or
+// what is computed from it.
+int finish(SolverImpl &s) {
+    int *flag = (int *)&s.pinned[62];
+    CU(cudaMemcpyAsync(flag, s.derr, sizeof(int), cudaMemcpyDeviceToHost, s.stream));
     CU(cudaStreamSynchronize(s.stream));
-    if (flag) {
+    if (*flag) {
         CU(cudaMemsetAsync(s.derr, 0, sizeof(int), s.stream));
         set_error("a bounded device wait timed out in the step kernel");
         return LBM_ETIMEOUT;
@@ -700,8 +702,7 @@ int lbm_solver_step(lbm_solver *h, int64_t n) {
 
 int lbm_solver_sync(lbm_solver *h) {
     if (!h) { set_error("NULL solver"); return LBM_EINVAL; }
-    CU(cudaStreamSynchronize(h->s.stream));
-    return check_device_error(h->s);
+    return finish(h->s);
 }
 
 int lbm_solver_get_f(lbm_solver *h, double *f) {
@@ -714,7 +715,7 @@ int lbm_solver_get_f(lbm_solver *h, double *f) {
         CU(cudaMemcpyAsync(f + a * n, s.stage, n * sizeof(double), cudaMemcpyDeviceToHost, s.stream));
         CU(cudaStreamSynchronize(s.stream));
     }
-    return LBM_OK;
+    return finish(s);
     API_END
 }
 
@@ -757,8 +758,7 @@ int lbm_solver_macros(lbm_solver *h, double *rho, double *ux, double *uy, double
     }));
     for (int i = 0; i < 4; ++i)
         if (hst[i]) CU(cudaMemcpyAsync(hst[i], d[i], n * sizeof(double), cudaMemcpyDeviceToHost, s.stream));
-    CU(cudaStreamSynchronize(s.stream));
-    return LBM_OK;
+    return finish(s);
     API_END
 }
 
@@ -782,8 +782,7 @@ int lbm_solver_macros_mean(lbm_solver *h, int64_t nsteps, double *rho, double *u
     double *hst[4] = {rho, ux, uy, T};
     for (int i = 0; i < 4; ++i)
         if (hst[i]) CU(cudaMemcpyAsync(hst[i], d[i], n * sizeof(double), cudaMemcpyDeviceToHost, s.stream));
-    CU(cudaStreamSynchronize(s.stream));
-    if (int rc = check_device_error(s)) return rc;
+    if (int rc = finish(s)) return rc;
     for (int i = 0; i < 4; ++i)
         if (hst[i])
             for (size_t c = 0; c < n; ++c) hst[i][c] /= (double)nsteps;
@@ -805,8 +804,7 @@ int lbm_solver_fluxes(lbm_solver *h, double *sxx, double *sxy, double *syy, doub
     }));
     for (int i = 0; i < 5; ++i)
         if (hst[i]) CU(cudaMemcpyAsync(hst[i], d[i], n * sizeof(double), cudaMemcpyDeviceToHost, s.stream));
-    CU(cudaStreamSynchronize(s.stream));
-    return LBM_OK;
+    return finish(s);
     API_END
 }
 
@@ -844,8 +842,7 @@ int lbm_solver_get_state(lbm_solver *h, void *buf, size_t bytes) {
     const size_t fb = (size_t)s.L.Q * s.p.Ny * s.nt * s.pitch * s.elem;
     CU(cudaMemcpyAsync(b + 64, s.f[s.cur], fb, cudaMemcpyDeviceToHost, s.stream));
     if (s.rho[0]) CU(cudaMemcpyAsync(b + 64 + fb, s.rho[s.cur], (size_t)s.p.Ny * s.nt * s.pitch * 4, cudaMemcpyDeviceToHost, s.stream));
-    CU(cudaStreamSynchronize(s.stream));
-    return LBM_OK;
+    return finish(s);
     API_END
 }
 
@@ -902,8 +899,7 @@ int lbm_solver_run_to_residual(lbm_solver *h, double tol, int64_t max_steps, int
         CU(launch_residual_partials(s.stream, s.stage + n, s.stage + 3 * n, s.prev, s.prev + n, n, Tref, s.red, nb));
         CU(launch_final_sum(s.stream, s.red, nb, 5, s.red + 8 * 1024));
         CU(cudaMemcpyAsync(s.pinned, s.red + 8 * 1024, 5 * sizeof(double), cudaMemcpyDeviceToHost, s.stream));
-        CU(cudaStreamSynchronize(s.stream));
-        if ((rc = check_device_error(s))) return rc;
+        if ((rc = finish(s))) return rc;
         const double *v = s.pinned;
         if (v[4] > 0) { status = LBM_ENONFINITE; r = NAN; break; }
         r = std::sqrt(v[0]) / std::fmax(std::sqrt(v[1]), 1e-30);
@@ -964,8 +960,7 @@ int lbm_solver_wall_mass(lbm_solver *h, double *m_in) {
     SolverImpl &s = h->s;
     CU(dispatch_prec(s.p.precision, [&](auto P) { return Launch<decltype(P)::value>::wall_mass(s, s.stage); }));
     CU(cudaMemcpyAsync(m_in, s.stage, 2 * (size_t)s.p.Nx * sizeof(double), cudaMemcpyDeviceToHost, s.stream));
-    CU(cudaStreamSynchronize(s.stream));
-    return LBM_OK;
+    return finish(s);
     API_END
 }
 
