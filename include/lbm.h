@@ -272,21 +272,21 @@ int lbm_solver_stats(lbm_solver *s, lbm_stats *st);
  * grid of several x-tiles). */
 int lbm_solver_set_kernel(lbm_solver *s, int32_t kernel, int32_t variant);
 
-/* Limit, in nanoseconds of the GPU's global timer, of each bounded wait of
- * the staged kernel (its mbarrier waits between the producer warp and the
- * consumer warps; default 2 s).  The paper has no counterpart: it is the
- * library's failure detection.  A wait that runs out records a device flag,
- * the CTA stops taking tiles and its producer waits for its copies in flight
- * (with a fixed 2 s limit of its own) before the CTA exits; the next
+/* Limit, in nanoseconds of the GPU's global timer, of each bounded wait
+ * (default 2 s): the staged kernel's mbarrier waits between the producer warp
+ * and the consumer warps, and the grid barrier between the steps that FP64
+ * CELLWARP grids of more than 64 cells advance in one launch.  The paper has
+ * no counterpart: it is the library's failure detection.  A wait that runs out
+ * records a device flag; a staged CTA stops taking tiles and its producer waits
+ * for its copies in flight (with a fixed 2 s limit of its own) before the CTA
+ * exits; the blocks behind a grid barrier take no further step.  The next
  * lbm_solver_sync, lbm_solver_run_to_residual or call that reads the state
  * out (get_f, get_state, macros, macros_mean, fluxes, wall_mass, stats)
  * returns LBM_ETIMEOUT and clears the flag.  The state of that step is then
  * incomplete: reload one (set_state, set_f or init) before stepping on.  0
  * makes every such wait give up at once, met or not (the failure path on
- * demand; the drain before exit still waits).  FP64 CELLWARP grids advance
- * many steps per launch behind a grid barrier whose waits have a fixed 2 s
- * limit and the same outcome; the other kernels have no waits.
- * Errors: LBM_EINVAL. */
+ * demand; the drain before exit still waits).  The other kernels have no
+ * bounded waits.  Errors: LBM_EINVAL. */
 int lbm_solver_set_wait_limit(lbm_solver *s, uint64_t ns);
 /* Number of compiled variants of `kernel` (DIRECT or STAGED) for this
  * solver's precision.  Errors: LBM_EINVAL. */

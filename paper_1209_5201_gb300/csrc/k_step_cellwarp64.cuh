@@ -308,8 +308,9 @@ k_steps_cellwarp64_cluster(const double *fin, double *fout,
 // is resident): the state alternates between the two buffers in global memory
 // (L2), a grid barrier separates the steps.  bar: [0] arrivals, [1] blocks
 // that have left, [2] a wait ran out; zero before and after every launch.
-// Each wait is bounded (2 s): on expiry the error flag is set and every block
-// leaves.  The halo copies are written by the last step only.
+// Each wait is bounded (KConsts::wait_ns; 0: gives up at once, met or not): on
+// expiry the error flag is set and every block leaves.  The halo copies are
+// written by the last step only.
 template <int Q, int MAXWARPS>
 __global__ void __launch_bounds__(32 * MAXWARPS, 1)
 k_steps_cellwarp64_grid(double *f0, double *f1, const __grid_constant__ KConsts<double> k,
@@ -355,10 +356,11 @@ k_steps_cellwarp64_grid(double *f0, double *f1, const __grid_constant__ KConsts<
             unsigned long long t0 = 0;
             for (int spin = 0;; ++spin) {
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(seen) : "l"(bar) : "memory");
-                if (seen >= goal) break;
-                if ((spin & 255) == 255) {
+                bool late = k.wait_ns == 0;
+                if (!late && seen >= goal) break;
+                if (late || (spin & 255) == 255) {
                     if (t0 == 0) t0 = global_ns();
-                    const bool late = global_ns() - t0 > kDefaultWaitNs;
+                    late = late || global_ns() - t0 > k.wait_ns;
                     if (late) {
                         atomicOr(err, kCellErrTimeout);
                         atomicExch(bar + 2, 1u);
@@ -373,10 +375,15 @@ k_steps_cellwarp64_grid(double *f0, double *f1, const __grid_constant__ KConsts<
         __syncthreads();
         if (s_stop) break;
     }
-    // the last block to leave clears the barrier for the next launch
-    if (threadIdx.x == 0 && atomicAdd(bar + 1, 1u) == gridDim.x - 1) {
-        bar[0] = bar[1] = bar[2] = 0u;
+    // the last block to leave clears the barrier for the next launch: every
+    // block's arrivals (one that gave up has not seen its own counted) come
+    // before its count here
+    if (threadIdx.x == 0) {
         __threadfence();
+        if (atomicAdd(bar + 1, 1u) == gridDim.x - 1) {
+            __threadfence();
+            bar[0] = bar[1] = bar[2] = 0u;
+        }
     }
 }
 

@@ -105,8 +105,9 @@ struct KConsts {
     // steps done when state buffer b (base f0 for b = 0) is the source
     const void *f0;
     unsigned *sr;
-    // limit of each bounded mbarrier wait of the staged kernel (ns); the
-    // wait for copies in flight before a CTA exits keeps its own fixed limit
+    // limit (ns) of each bounded wait: the staged kernel's mbarriers, the grid
+    // barrier of the many-step FP64 kernel; the staged wait for copies in flight
+    // before a CTA exits keeps its own fixed limit
     unsigned long long wait_ns;
 };
 

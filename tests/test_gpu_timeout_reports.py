@@ -56,3 +56,14 @@ def test_staged_timeout_is_reported_by_every_read_out(lbm, call):
     for s in (a, b):
         s.set_kernel(lbm.LBM_KERNEL_STAGED, 0)
     _expire_and_recover(lbm, a, b, READ_OUTS[call], inputs.rho_field(70, 12, 1e-2, seed=8), (5,))
+
+
+# more than 64 cells: the whole-chip launch with a grid barrier, one block to many
+@pytest.mark.parametrize("Nx,Ny", [(5, 13), (1, 500), (60, 60)])
+def test_fp64_grid_barrier_wait_limit(lbm, Nx, Ny):
+    a, b = _solvers(lbm, 2, Nx=Nx, Ny=Ny)
+    for s in (a, b):
+        s.set_kernel(lbm.LBM_KERNEL_CELLWARP)
+    # several launches afterwards: the barrier's words were left as it needs them
+    _expire_and_recover(lbm, a, b, READ_OUTS["macros"], inputs.rho_field(Nx, Ny, 1e-2, seed=8),
+                        (7, 2, 33, 2100))
