@@ -367,6 +367,12 @@ int launch_step_variant(SolverImpl &s, int src, int dst, int kernel, int variant
     });
 }
 
+int launch_many_steps(SolverImpl &s, int n) {
+    return dispatch_prec(s.p.precision, [&](auto P) {
+        return Launch<decltype(P)::value>::steps_cellwarp(s, s.cur, n);
+    });
+}
+
 }  // namespace lbm
 
 using namespace lbm;
@@ -676,9 +682,7 @@ int lbm_solver_step(lbm_solver *h, int64_t n) {
     int rc;
     while (n >= 2 && kern == LBM_KERNEL_CELLWARP) {
         const int m = (int)std::min<int64_t>(n, kLaunchSteps);
-        const int e = dispatch_prec(s.p.precision, [&](auto P) {
-            return Launch<decltype(P)::value>::steps_cellwarp(s, s.cur, m);
-        });
+        const int e = launch_many_steps(s, m);
         if (e == (int)cudaErrorNotSupported) break;
         CU(e);
         s.cur ^= m & 1;

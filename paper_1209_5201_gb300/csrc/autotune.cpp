@@ -7,6 +7,7 @@
 // Results are cached per (lattice, precision, order, Nx class, Ny class) for
 // the life of the process and, when LBM_AUTOTUNE_CACHE names a file, across
 // processes (one "key kernel variant ms" line per class).
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <map>
@@ -65,20 +66,31 @@ void append_file_cache(const std::string &key, const Choice &c) {
     std::fclose(fh);
 }
 
+// n steps by the launches lbm_solver_step makes: of the one-warp-per-cell kernel
+// many steps in one where it has such a launch
+int enqueue(SolverImpl &s, int kernel, int variant, int n) {
+    while (n >= 2 && kernel == LBM_KERNEL_CELLWARP) {
+        const int m = std::min(n, kLaunchSteps);
+        const int e = launch_many_steps(s, m);
+        if (e == (int)cudaErrorNotSupported) break;
+        if (e) return LBM_ECUDA;
+        s.cur ^= m & 1;
+        n -= m;
+    }
+    for (int i = 0; i < n; ++i) {
+        if (launch_step_variant(s, s.cur, s.cur ^ 1, kernel, variant)) return LBM_ECUDA;
+        s.cur ^= 1;
+    }
+    return LBM_OK;
+}
+
 int time_candidate(SolverImpl &s, int kernel, int variant, int trial, double *ms) {
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess) return LBM_ECUDA;
     if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return LBM_ECUDA; }
-    int rc = LBM_OK;
-    for (int i = 0; i < 2 && !rc; ++i) {
-        if (launch_step_variant(s, s.cur, s.cur ^ 1, kernel, variant)) rc = LBM_ECUDA;
-        s.cur ^= 1;
-    }
+    int rc = enqueue(s, kernel, variant, 2);
     cudaEventRecord(e0, s.stream);
-    for (int i = 0; i < trial && !rc; ++i) {
-        if (launch_step_variant(s, s.cur, s.cur ^ 1, kernel, variant)) rc = LBM_ECUDA;
-        s.cur ^= 1;
-    }
+    if (!rc) rc = enqueue(s, kernel, variant, trial);
     cudaEventRecord(e1, s.stream);
     float t = 0;
     if (!rc && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&t, e0, e1) == cudaSuccess)

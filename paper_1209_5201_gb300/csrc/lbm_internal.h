@@ -214,6 +214,9 @@ TileLayout tile_layout(int Nx, int precision);
 int staged_variant_count(int precision);
 int direct_variant_count(int precision);
 int launch_step_variant(SolverImpl &s, int src, int dst, int kernel, int variant);
+// n >= 2 (at most kLaunchSteps) steps of the one-warp-per-cell kernel from the
+// current buffer in one launch; cudaErrorNotSupported where it has none
+int launch_many_steps(SolverImpl &s, int n);
 // Re-initialise the state as lbm_solver_init does (rest equilibrium + noise).
 int dispatch_init_rest(SolverImpl &s);
 // Pick the fastest step kernel / variant for this solver (autotune.cpp).

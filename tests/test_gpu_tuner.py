@@ -1,0 +1,42 @@
+"""The autotuner's choice against the candidates it chose from."""
+import pytest
+
+from gpu_util import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    return need_gpu()
+
+
+def _us(s, n, best_of=5):
+    import torch
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    s.step(n)
+    us = []
+    for _ in range(best_of):
+        e0.record(s.stream)
+        s.step(n)
+        e1.record(s.stream)
+        e1.synchronize()
+        us.append(e0.elapsed_time(e1) * 1e3 / n)
+    return min(us)
+
+
+def _solver(lbm, **kw):
+    import torch
+    args = dict(lattice="D2Q37", eq_order=3, thermal=True, Kn=0.06, u_wall=(-0.2, 0.2), noise_amp=1e-3)
+    return lbm.Solver(lbm.Config(**{**args, **kw}), stream=torch.cuda.Stream())
+
+
+def test_fp64_tuner_times_the_many_step_launches(lbm):
+    # one launch per step 19 us, many per launch 13, one thread per cell 18
+    s = _solver(lbm, Nx=50, Ny=60, precision="fp64")
+    s.autotune(10)
+    tuned = _us(s, 400)
+    s.set_kernel(lbm.LBM_KERNEL_CELLWARP)
+    warp = _us(s, 400)
+    s.close()
+    assert tuned <= 1.15 * warp
