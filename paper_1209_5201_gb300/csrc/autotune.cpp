@@ -2,8 +2,9 @@
 //
 // Candidates: every variant of the one-pass direct kernel and of the TMA-staged one compiled
 // for the solver's precision, which round alike; in FP64 also the one-warp-per-cell kernel.
-// FP32 and BF16 grids take the latter by size alone (cellwarp_cells).  Each runs `trial` steps after two warm-up
-// steps, timed with CUDA events on the solver's stream; the fastest wins.
+// FP32 and BF16 grids take the latter by size alone (cellwarp_by_size).  Each runs
+// `trial` steps after two warm-up steps, timed with CUDA events on the solver's
+// stream; the fastest wins.
 // Results are cached per (lattice, precision, order, Nx class, Ny class) for
 // the life of the process and, when LBM_AUTOTUNE_CACHE names a file, across
 // processes (one "key kernel variant ms" line per class).
@@ -102,30 +103,35 @@ int time_candidate(SolverImpl &s, int kernel, int variant, int trial, double *ms
     return rc;
 }
 
-// Cells up to which a tuned FP32 or BF16 grid takes the one-warp-per-cell
-// kernel.  That kernel sums the moments in another order than the others, so
-// the choice shows in the results (at FP32 round-off; in BF16 through the
-// rounding of what is stored) and is made by size, not by a timing that differs
-// from run to run.  The line lies where it was the faster one (us per step on
-// square grids, one warp per cell / one thread per cell): FP32 D2Q37 16 / 16.6 at
-// 6000 cells, 17 / 16.7 at 7000; D2Q25 12.3 / 12.5 at 5000; D2Q17 never; BF16DEV
-// D2Q37 26 / 27 at 12 000, D2Q25 18.4 / 18.7 at 10 000; BF16SHIFT D2Q37 22 / 25 at
-// 10 000, D2Q25 15.8 / 17.3 at 8000.  (The one-thread kernels' wall rows have
-// become three times faster since; moving the line would change results.)
-long long cellwarp_cells(int Q, int precision) {
-    const int i = Q == 37 ? 0 : Q == 25 ? 1 : 2;
-    constexpr long long fp32[3] = {6500, 4800, 0}, dev[3] = {13000, 9700, 3700},
-                        shift[3] = {11000, 9000, 2700};
-    return precision == LBM_FP32 ? fp32[i] : precision == LBM_BF16DEV ? dev[i] : shift[i];
+// Whether a tuned FP32 or BF16 grid takes the one-warp-per-cell kernel.  That
+// kernel sums the moments in another order than the others, so the choice shows
+// in the results (at FP32 round-off; in BF16 through the rounding of what is
+// stored): it is made by size, not by a timing that differs from run to run, and
+// the line is not moved with the kernels' speeds, for that would change the
+// results of grids in use.  (Below it the one-thread kernels are the faster ones
+// in FP32: D2Q37 60 x 60 4.0 us per step, one warp per cell 11.2; set_kernel
+// takes either.)  Cells of a grid of fewer and of kWideColumns or more columns:
+// a wide grid has more wall rows to its cells, whose warps sum the incoming mass
+// of seven ghost columns first.
+constexpr int kWideColumns = 120;
+bool cellwarp_by_size(const SolverImpl &s) {
+    struct Line { long long narrow, wide; };
+    constexpr Line fp32[3] = {{6500, 4100}, {4800, 2200}, {0, 0}},
+                   dev[3] = {{13000, 13000}, {9700, 9700}, {3700, 3700}},
+                   shift[3] = {{11000, 11000}, {9000, 9000}, {2700, 2200}};
+    if (s.p.precision == LBM_FP64) return false;
+    const int i = s.L.Q == 37 ? 0 : s.L.Q == 25 ? 1 : 2;
+    const Line l = s.p.precision == LBM_FP32 ? fp32[i] : s.p.precision == LBM_BF16DEV ? dev[i] : shift[i];
+    return (long long)s.p.Nx * s.p.Ny <= (s.p.Nx < kWideColumns ? l.narrow : l.wide);
 }
 
 }  // namespace
 
 int autotune_solver(SolverImpl &s, int trial) {
-    const std::string key = class_key(s);
     const long long cells = (long long)s.p.Nx * s.p.Ny;
     const bool by_size = s.p.precision != LBM_FP64;
-    const bool small = by_size && cells <= cellwarp_cells(s.L.Q, s.p.precision);
+    const bool small = cellwarp_by_size(s);
+    const std::string key = class_key(s);
     {
         // (a size class may straddle the line: the other kernel's entry is not its)
         std::lock_guard<std::mutex> lk(g_mu);

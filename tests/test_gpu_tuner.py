@@ -40,3 +40,19 @@ def test_fp64_tuner_times_the_many_step_launches(lbm):
     warp = _us(s, 400)
     s.close()
     assert tuned <= 1.15 * warp
+
+
+# wide grids below the line by cells, where one warp per cell is the slower kernel
+@pytest.mark.parametrize("lattice,Nx,Ny,precision", [
+    ("D2Q37", 122, 41, "fp32"), ("D2Q37", 224, 22, "fp32"), ("D2Q37", 212, 21, "fp32"),
+    ("D2Q25", 200, 20, "fp32"), ("D2Q17", 141, 16, "bf16shift")])
+def test_wide_grids_are_not_held_on_the_slower_kernel(lbm, lattice, Nx, Ny, precision):
+    o, t = (3, True) if lattice == "D2Q37" else (2, False)
+    s = _solver(lbm, lattice=lattice, Nx=Nx, Ny=Ny, precision=precision, eq_order=o, thermal=t)
+    s.autotune(10)
+    tuned = _us(s, 400)
+    s.set_kernel(lbm.LBM_KERNEL_DIRECT)
+    direct = _us(s, 400)
+    s.close()
+    assert tuned <= 1.25 * direct
+
