@@ -295,11 +295,12 @@ int lbm_solver_variant_count(lbm_solver *s, int32_t kernel, int32_t *n);
  * variants. */
 int lbm_solver_kernel_info(lbm_solver *s, int32_t *kernel, int32_t *variant,
                            int32_t *nvariants);
-/* Autotuner: time trial_steps steps of every direct and every staged
- * variant (FP64: and of the one-warp-per-cell kernel; FP32 and BF16 grids of a
- * few thousand cells take that one by size) on this solver's grid (CUDA events on the solver's stream), keep
- * the fastest, and cache the choice per (lattice, precision, order, Nx and Ny
- * rounded up to powers of two) for the process, and in the file named by the
+/* Autotuner: time trial_steps steps of every direct and every staged variant
+ * (FP64: and of the one-warp-per-cell kernel; FP32 and BF16 grids of a few
+ * thousand cells take that one by size) on this solver's grid (CUDA events on
+ * the solver's stream), keep the fastest, and cache the choice per (lattice,
+ * precision, order, Nx and Ny rounded up to powers of two, and whether the grid
+ * is one that takes its kernel by size) for the process, and in the file named by the
  * environment variable LBM_AUTOTUNE_CACHE when set.  Overwrites the state:
  * on return the solver holds the lbm_solver_init state.  Synchronous.
  * Errors: LBM_EINVAL, LBM_ECUDA. */

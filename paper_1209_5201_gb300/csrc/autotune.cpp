@@ -131,9 +131,9 @@ int autotune_solver(SolverImpl &s, int trial) {
     const long long cells = (long long)s.p.Nx * s.p.Ny;
     const bool by_size = s.p.precision != LBM_FP64;
     const bool small = cellwarp_by_size(s);
-    const std::string key = class_key(s);
+    // a size class may straddle the line: an entry for each side
+    const std::string key = class_key(s) + (small ? "_w" : "");
     {
-        // (a size class may straddle the line: the other kernel's entry is not its)
         std::lock_guard<std::mutex> lk(g_mu);
         load_file_cache();
         auto it = g_cache.find(key);

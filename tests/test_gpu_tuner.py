@@ -56,3 +56,11 @@ def test_wide_grids_are_not_held_on_the_slower_kernel(lbm, lattice, Nx, Ny, prec
     s.close()
     assert tuned <= 1.25 * direct
 
+
+def test_a_size_class_across_the_line_keeps_both_choices(lbm):
+    # 70 x 60 and 128 x 64: one class, on either side of the line
+    small = _solver(lbm, Nx=70, Ny=60, precision="fp32")
+    large = _solver(lbm, Nx=128, Ny=64, precision="fp32")
+    first = small.autotune(10), large.autotune(10)
+    assert (small.autotune(10), large.autotune(10)) == first
+    small.close(), large.close()
