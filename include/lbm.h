@@ -259,8 +259,8 @@ int lbm_solver_stats(lbm_solver *s, lbm_stats *st);
 
 /* Step-kernel selection.  LBM_KERNEL_DIRECT: one thread per cell, populations
  * pulled straight from global memory; its variants differ in block width,
- * register cap (variant 0: by format and lattice), rows per block and store
- * cache policy.  LBM_KERNEL_STAGED: persistent tile
+ * register cap (variant 0: by format and lattice; the last one of FP32 and
+ * BF16: none, which is FP64's variant 0), rows per block and store cache policy.  LBM_KERNEL_STAGED: persistent tile
  * kernel whose producer warp stages each velocity's shifted source window
  * (tile plus the +-3-cell halo, rounded to 16 bytes in x) into shared memory
  * with TMA; `variant` picks one of the compiled tile shapes, 0 <= variant <

@@ -354,6 +354,12 @@ int direct_variant_count(int precision) {
     return dispatch_prec(precision, [&](auto P) { return Launch<decltype(P)::value>::direct_variants(); });
 }
 
+bool direct_variant_repeats(const SolverImpl &s, int variant) {
+    return dispatch_prec(s.p.precision, [&](auto P) {
+        return (int)Launch<decltype(P)::value>::direct_repeats(s.L.Q, variant);
+    }) != 0;
+}
+
 int dispatch_init_rest(SolverImpl &s) {
     return init_state(s, nullptr, nullptr, nullptr, nullptr);
 }

@@ -1,7 +1,8 @@
 // Tile / block-shape autotuner of the step kernel.
 //
-// Candidates: every variant of the one-pass direct kernel and of the TMA-staged one compiled
-// for the solver's precision, which round alike; in FP64 also the one-warp-per-cell kernel.
+// Candidates: every variant of the one-pass direct kernel (variant 0's once, though the
+// same request may be listed again) and of the TMA-staged one compiled for the solver's
+// precision, which round alike; in FP64 also the one-warp-per-cell kernel.
 // FP32 and BF16 grids take the latter by size alone (cellwarp_by_size).  Each runs
 // `trial` steps after two warm-up steps, timed with CUDA events on the solver's
 // stream; the fastest wins.
@@ -152,6 +153,7 @@ int autotune_solver(SolverImpl &s, int trial) {
     double ms = 0;
     const int nd = small ? 0 : direct_variant_count(s.p.precision);
     for (int v = 0; v < nd; ++v) {
+        if (direct_variant_repeats(s, v)) continue;
         if ((rc = time_candidate(s, LBM_KERNEL_DIRECT, v, trial, &ms))) return rc;
         if (ms < best.ms) best = Choice{LBM_KERNEL_DIRECT, v, ms};
     }

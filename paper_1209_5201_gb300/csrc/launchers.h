@@ -10,6 +10,8 @@ template <int PREC>
 struct Launch {
     static int step(SolverImpl &s, int src, int dst, int variant);   // direct kernel
     static int direct_variants();
+    // whether a variant above 0 is variant 0's kernel again on this lattice
+    static bool direct_repeats(int Q, int variant);
     static int step_staged(SolverImpl &s, int src, int dst, int variant);
     static int step_cellwarp(SolverImpl &s, int src, int dst);
     // n steps in one launch; cudaErrorNotSupported: use step_cellwarp

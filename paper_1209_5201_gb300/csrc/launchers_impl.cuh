@@ -51,9 +51,10 @@ inline int aux_blocks(long long n) {
 // ---- direct kernel variants {BX, MINB, CS, RS} ----------------------------------
 // RS: rows per block.  MINB < 0: the format's own choice (default_blocks).
 struct DirectVariants {
-    static constexpr int n = 8;
+    static constexpr int n = 9;
     static constexpr int v[n][4] = {{128, -1, 0, 1}, {128, 7, 0, 1}, {128, 6, 0, 1}, {256, 0, 0, 1},
-                                    {128, 0, 1, 1}, {192, 0, 0, 1}, {128, 0, 0, 2}, {128, 5, 0, 1}};
+                                    {128, 0, 1, 1}, {192, 0, 0, 1}, {128, 0, 0, 2}, {128, 5, 0, 1},
+                                    {128, 0, 0, 1}};
 };
 // Blocks per SM that variant 0 asks the register allocator for, by what
 // measured fastest untuned, us per step on 4096 x 2048 / 2050 x 1023 /
@@ -139,6 +140,7 @@ int step_q(SolverImpl &s, int src, int dst, int variant) {
         LBM_DIRECT_CASE(5)
         LBM_DIRECT_CASE(6)
         LBM_DIRECT_CASE(7)
+        LBM_DIRECT_CASE(8)
     default: break;
     }
 #undef LBM_DIRECT_CASE
@@ -157,7 +159,20 @@ int Launch<PREC>::step(SolverImpl &s, int src, int dst, int variant) {
 }
 
 template <int PREC>
-int Launch<PREC>::direct_variants() { return DirectVariants::n; }
+int Launch<PREC>::direct_variants() {
+    // the last shape, no request, is FP64's variant 0
+    return PREC == LBM_FP64 ? DirectVariants::n - 1 : DirectVariants::n;
+}
+
+template <int PREC>
+bool Launch<PREC>::direct_repeats(int Q, int variant) {
+    using V = DirectVariants;
+    const int blocks = Q == 37   ? default_blocks<37, PREC>()
+                       : Q == 25 ? default_blocks<25, PREC>()
+                                 : default_blocks<17, PREC>();
+    return variant > 0 && V::v[variant][0] == V::v[0][0] && V::v[variant][1] == blocks &&
+           V::v[variant][2] == V::v[0][2] && V::v[variant][3] == V::v[0][3];
+}
 
 template <int PREC>
 int Launch<PREC>::step_cellwarp(SolverImpl &s, int src, int dst) {

@@ -213,6 +213,7 @@ struct TileLayout {
 TileLayout tile_layout(int Nx, int precision);
 int staged_variant_count(int precision);
 int direct_variant_count(int precision);
+bool direct_variant_repeats(const SolverImpl &s, int variant);   // variant 0's kernel again
 int launch_step_variant(SolverImpl &s, int src, int dst, int kernel, int variant);
 // n >= 2 (at most kLaunchSteps) steps of the one-warp-per-cell kernel from the
 // current buffer in one launch; cudaErrorNotSupported where it has none

@@ -6,4 +6,5 @@ namespace lbm {
 extern template int step_q<LBM_BF16SHIFT, 37>(SolverImpl &, int, int, int);
 template int Launch<LBM_BF16SHIFT>::step(SolverImpl &, int, int, int);
 template int Launch<LBM_BF16SHIFT>::direct_variants();
+template bool Launch<LBM_BF16SHIFT>::direct_repeats(int, int);
 }  // namespace lbm

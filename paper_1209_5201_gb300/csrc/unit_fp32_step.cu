@@ -6,4 +6,5 @@ namespace lbm {
 extern template int step_q<LBM_FP32, 37>(SolverImpl &, int, int, int);
 template int Launch<LBM_FP32>::step(SolverImpl &, int, int, int);
 template int Launch<LBM_FP32>::direct_variants();
+template bool Launch<LBM_FP32>::direct_repeats(int, int);
 }  // namespace lbm

@@ -1,4 +1,5 @@
 """The autotuner's choice against the candidates it chose from."""
+import numpy as np
 import pytest
 
 from gpu_util import need_gpu
@@ -64,3 +65,20 @@ def test_a_size_class_across_the_line_keeps_both_choices(lbm):
     first = small.autotune(10), large.autotune(10)
     assert (small.autotune(10), large.autotune(10)) == first
     small.close(), large.close()
+
+
+@pytest.mark.parametrize("precision,n", [("fp64", 8), ("fp32", 9), ("bf16dev", 9), ("bf16shift", 9)])
+@pytest.mark.parametrize("lattice,Nx", [("D2Q37", 300), ("D2Q37", 600), ("D2Q25", 300)])
+def test_the_shape_without_a_register_request_is_a_variant(lbm, precision, n, lattice, Nx):
+    # FP32 and BF16 variant 0 asks for registers by format and lattice; the
+    # shape that asks for none is the last variant, the same step bit for bit
+    o, t = (3, True) if lattice == "D2Q37" else (2, False)
+    a, b = (_solver(lbm, lattice=lattice, Nx=Nx, Ny=20, precision=precision, eq_order=o, thermal=t)
+            for _ in range(2))
+    assert a.variant_count(lbm.LBM_KERNEL_DIRECT) == n
+    for s, v in ((a, 0), (b, n - 1)):
+        s.set_kernel(lbm.LBM_KERNEL_DIRECT, v)
+        s.init()
+        s.step(20)
+    assert np.array_equal(a.get_f(), b.get_f())
+    a.close(), b.close()
