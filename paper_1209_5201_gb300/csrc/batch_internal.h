@@ -23,9 +23,18 @@ constexpr int kMaxTerm = 28;
 // sub), and more, up to kMaxLaunchChunks, while they fit the launch's time.
 constexpr int kMaxSub = 16;
 constexpr int kMaxLaunchChunks = 256;
-// A launch lasts as long as its slowest slot, at least about this (ns): the
-// host's work per launch is 20 - 50 us.
+// While nothing waits for its end, a launch goes on for about this long (ns):
+// the host's work per launch is 20 - 50 us.
 constexpr unsigned long long kMinLaunchNs = 2000000ull;
+// How long a launch may last (device memory, uploaded with each launch).  Slots
+// run further chunks up to `base`, the time the slowest of them takes for its
+// own chunks anyway, and up to `more` as long as no slot has stopped in this
+// launch (its result is read out at the launch's end) and the host has not
+// raised its word (a request has arrived or is to be cancelled).
+struct LaunchBudget {
+    unsigned long long base, more;
+    int stopped;              // set by the kernels
+};
 // Chunks per launch of a slot on a cluster of cl CTAs: about the factor by
 // which the cluster shortens a step of a tall column, conservatively, so that
 // a cluster slot is rarely the one a launch waits for.
@@ -126,11 +135,11 @@ int batch_max_cluster();
 // dbg: 8 device ints; dbg[0] != 0 records the first invalid descriptor or
 // read-out offset a kernel met (and skipped).
 // Chunks of the slots [slot0, slot0 + nlanes), each on a cluster of CL CTAs;
-// budget: device word with the time (ns) the launch may take anyway; part: kMaxResidualChunks x 6 FP64 residual partials per slot of the
-// whole table.
+// waiting: the host's word (pinned memory), see LaunchBudget; part:
+// kMaxResidualChunks x 6 FP64 residual partials per slot of the whole table.
 int launch_batch_chunk(cudaStream_t st, SlotDesc *desc, SlotStatus *status, float *pool,
                        double *part, int slot0, int nlanes, int CL, long long pool_elems,
-                       const unsigned long long *budget, int *dbg);
+                       LaunchBudget *budget, const int *waiting, int *dbg);
 int launch_batch_init(cudaStream_t st, SlotDesc *desc, float *pool, const int *slots, int n,
                       float rho0, int nslots, long long pool_elems, int *dbg);
 int launch_batch_macros(cudaStream_t st, const SlotDesc *desc, const float *pool,

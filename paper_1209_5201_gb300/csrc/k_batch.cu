@@ -60,10 +60,11 @@ __device__ __forceinline__ void load_desc(const SlotDesc *g, SlotDesc *s) {
 __global__ void __launch_bounds__(kBatchThreads, 2)
 k_batch_chunk(SlotDesc *__restrict__ desc, SlotStatus *__restrict__ status,
               float *__restrict__ pool, double *__restrict__ part, int slot0, int CL,
-              long long pool_elems, const unsigned long long *__restrict__ budget, int *dbg) {
+              long long pool_elems, LaunchBudget *budget, const int *waiting, int *dbg) {
     const unsigned long long t0 = global_ns();
     __shared__ SlotDesc sd;
     __shared__ BatchWallShared sw;
+    __shared__ LaunchTime lt;
     __shared__ int s_chunks, s_precise;
     __shared__ long long s_steps;
     extern __shared__ __align__(16) float batch_sm[];
@@ -74,6 +75,7 @@ k_batch_chunk(SlotDesc *__restrict__ desc, SlotStatus *__restrict__ status,
         s_chunks = status[slot].chunks;
         s_steps = status[slot].steps;
         s_precise = status[slot].precise;
+        lt = LaunchTime{t0, budget->base, budget->more, 0, &budget->stopped, waiting};
     }
     __syncthreads();
     if (sd.Q == 0 || status[slot].state != kSlotRunning) return;
@@ -81,9 +83,9 @@ k_batch_chunk(SlotDesc *__restrict__ desc, SlotStatus *__restrict__ status,
     double *pp = part + (long long)slot * (6 * kMaxResidualChunks);
     int done = 0;
     switch (sd.Q) {
-    case 17: done = batch_slot<17>(sd, pool, status + slot, sw, rank, CL, s_chunks, s_steps, s_precise, pp, batch_sm, t0, *budget); break;
-    case 25: done = batch_slot<25>(sd, pool, status + slot, sw, rank, CL, s_chunks, s_steps, s_precise, pp, batch_sm, t0, *budget); break;
-    case 37: done = batch_slot<37>(sd, pool, status + slot, sw, rank, CL, s_chunks, s_steps, s_precise, pp, batch_sm, t0, *budget); break;
+    case 17: done = batch_slot<17>(sd, pool, status + slot, sw, rank, CL, s_chunks, s_steps, s_precise, pp, batch_sm, lt); break;
+    case 25: done = batch_slot<25>(sd, pool, status + slot, sw, rank, CL, s_chunks, s_steps, s_precise, pp, batch_sm, lt); break;
+    case 37: done = batch_slot<37>(sd, pool, status + slot, sw, rank, CL, s_chunks, s_steps, s_precise, pp, batch_sm, lt); break;
     default: break;
     }
     // the global-memory path leaves the state in the other buffer after an odd
@@ -227,11 +229,11 @@ int batch_max_cluster() {
 
 int launch_batch_chunk(cudaStream_t st, SlotDesc *desc, SlotStatus *status, float *pool,
                        double *part, int slot0, int nlanes, int CL, long long pool_elems,
-                       const unsigned long long *budget, int *dbg) {
+                       LaunchBudget *budget, const int *waiting, int *dbg) {
     if (nlanes <= 0) return 0;
     if (CL == 1) {
         k_batch_chunk<<<nlanes, kBatchThreads, kSmemBytes, st>>>(desc, status, pool, part, slot0,
-                                                                 1, pool_elems, budget, dbg);
+                                                                 1, pool_elems, budget, waiting, dbg);
         return (int)cudaGetLastError();
     }
     if (CL != 2 && CL != 4 && CL != 8 && CL != 16) return (int)cudaErrorInvalidValue;
@@ -248,7 +250,7 @@ int launch_batch_chunk(cudaStream_t st, SlotDesc *desc, SlotStatus *status, floa
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return (int)cudaLaunchKernelEx(&cfg, k_batch_chunk, desc, status, pool, part, slot0, CL,
-                                   pool_elems, budget, dbg);
+                                   pool_elems, budget, waiting, dbg);
 }
 
 int launch_batch_init(cudaStream_t st, SlotDesc *desc, float *pool, const int *slots, int n,

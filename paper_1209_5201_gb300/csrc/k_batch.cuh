@@ -33,6 +33,32 @@
 
 namespace lbm {
 
+// A launch's time as its CTAs hold it: when this one began, LaunchBudget's limits
+// and words, and from when on the words are read again (a read of host memory
+// takes about 4 us: one per chunk cost a lone 4096-row column 0.5 %).
+constexpr unsigned long long kLookNs = 300000ull;
+struct LaunchTime {
+    unsigned long long t0, base, more, look;
+    volatile int *stopped;
+    const volatile int *waiting;
+};
+
+// After chunk `done` of a slot's launch: whether another one ends in time (st->go).
+// Out of line: once per chunk, and its registers are not the step loop's.
+__device__ __noinline__ void launch_goes_on(LaunchTime &lt, SlotStatus *st, int sub, int done) {
+    const unsigned long long el = global_ns() - lt.t0, end = el + el / (unsigned)done;
+    if (done == sub) st->first_ns = (long long)el;
+    bool go = end <= lt.base;
+    if (!go && end <= lt.more) {
+        go = true;
+        if (el >= lt.look) {
+            go = (*lt.stopped | *lt.waiting) == 0;
+            lt.look = el + kLookNs;
+        }
+    }
+    st->go = go && done < kMaxLaunchChunks;
+}
+
 // Shared per-step wall data of a slot: the re-emitted deviations of Eq. (12)
 // per wall and velocity, the accommodation of each wall in FP32, and (state in
 // global memory) the post-collision values of the 3 rows next to each wall,
@@ -499,8 +525,7 @@ __device__ __forceinline__ void run_steps(const SlotDesc &d, State &S, BatchWall
 
 // The chunks of one launch for one slot on CTA `rank` of its CL-CTA cluster:
 // d.sub of them, and then more while another one, as long as those so far,
-// ends before `budget` ns from t0 - the time the slowest slot of the last launch
-// took, for which this launch lasts anyway (fewer when the slot stops:
+// ends within the launch's time (LaunchBudget; fewer when the slot stops:
 // converged, stagnated, non-finite or at max_steps); returns the chunks run.
 // Results do not depend on how many chunks a launch runs: 128 mixed columns on
 // 304 CTAs, whose tall one-CTA columns take 2.3 ms per chunk and clusters 0.2 -
@@ -515,7 +540,7 @@ __device__ __forceinline__ int batch_slot(const SlotDesc &d, float *__restrict__
                                           SlotStatus *__restrict__ st, BatchWallShared &sw,
                                           int rank, int CL, int chunks0, long long steps0,
                                           int precise, double *__restrict__ part, float *sm,
-                                          unsigned long long t0, unsigned long long budget) {
+                                          LaunchTime &lt) {
     using L = Lat<Q>;
     const int chunk = d.chunk_steps;
     const KConsts<float> &k = d.k;
@@ -693,13 +718,15 @@ __device__ __forceinline__ int batch_slot(const SlotDesc &d, float *__restrict__
     // one more chunk in this launch?  (the same answer in every thread of the cluster)
     auto another = [&](int done) -> bool {
         if (done < d.sub) return true;
-        if (rank == 0 && tid == 0) {
-            const unsigned long long el = global_ns() - t0;
-            if (done == d.sub) st->first_ns = (long long)el;
-            st->go = done < kMaxLaunchChunks && el + el / (unsigned)done <= budget;
-        }
+        if (rank == 0 && tid == 0) launch_goes_on(lt, st, d.sub, done);
         slot_barrier(CL);
         return __ldcg(&st->go) != 0;
+    };
+    // after chunk `done` of this launch: its check, then whether to go on
+    auto go_on = [&](auto &&at, int done) -> bool {
+        if (after_chunk(at, done)) return another(done);
+        if (rank == 0 && tid == 0) *lt.stopped = 1;
+        return false;
     };
 
     float *g_cur = pool + d.f_off + (d.cur ? (long long)Q * Ny : 0);
@@ -729,7 +756,7 @@ __device__ __forceinline__ int batch_slot(const SlotDesc &d, float *__restrict__
                 const int sl = RING ? (r - e * t) & (kRing - 1) : t * (kRing / 2) + r;
                 return sm + sl * Q + a;
             };
-            if (!after_chunk(at, done) || !another(done)) break;
+            if (!go_on(at, done)) break;
         }
         // write the final state back to the pool buffer it came from
         StaticFor<0, Q>::run([&](auto ic) {
@@ -754,7 +781,7 @@ __device__ __forceinline__ int batch_slot(const SlotDesc &d, float *__restrict__
             auto at = [=](int a, int, int r) -> float * {
                 return const_cast<float *>(src) + (long long)a * Ny + j0 + r;
             };
-            if (!after_chunk(at, done) || !another(done)) break;
+            if (!go_on(at, done)) break;
         }
     }
     return done;

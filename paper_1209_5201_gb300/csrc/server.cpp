@@ -111,9 +111,10 @@ struct ServerImpl {
     long long *d_off = nullptr;
     int *d_dbg = nullptr;                    // kernels' record of a rejected descriptor
     int *h_dbg = nullptr;
-    // time of the slowest running slot's part of the last launch: the others
-    // run further chunks within it
-    unsigned long long *d_budget = nullptr, *h_budget = nullptr;
+    LaunchBudget *d_budget = nullptr, *h_budget = nullptr;
+    // raised by submit and cancel, lowered when the worker has taken them up;
+    // the chunk kernels read it (pinned)
+    volatile int *h_waiting = nullptr;
     double *d_out = nullptr;                 // read-out staging
     long long out_elems = 0;
     // host mirrors (pinned)
@@ -393,7 +394,7 @@ struct ServerImpl {
             if (e == cudaSuccess)
                 e = (cudaError_t)launch_batch_chunk(side[c], d_desc, d_status, pool, d_part,
                                                     cls_base[c], cls_cap[c], kBatchClassCL[c],
-                                                    pool_elems, d_budget, d_dbg);
+                                                    pool_elems, d_budget, (const int *)h_waiting, d_dbg);
             if (e == cudaSuccess) e = cudaEventRecord(ev_join[c], side[c]);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev_join[c], 0);
         }
@@ -498,13 +499,34 @@ struct ServerImpl {
         return e;
     }
 
+    // The time of the next launch.  Beyond that of its slowest slot it goes on
+    // only while no request is queued and none of several running ones reaches
+    // its step limit within it: that one would wait for chunks the others have
+    // begun (a 256-row request of 2000 steps beside a long one: 4.3 ms with
+    // launches of one chunk, 4.6 - 4.9 with launches of 2 ms throughout).
+    LaunchBudget launch_budget(bool queued) const {
+        unsigned long long base = 0;
+        bool more = !queued;
+        for (int s = 0; s < (int)slots.size(); ++s) {
+            if (!slots[s].busy || h_status[s].state != kSlotRunning) continue;
+            const SlotDesc &d = h_desc[s];
+            const double ns = (double)h_status[s].first_ns;   // 0: not yet run
+            base = std::max(base, (unsigned long long)ns);
+            const double left = ns * (double)(d.max_steps - h_status[s].steps) / ((double)d.sub * d.chunk_steps);
+            if (running > 1 && left < (double)kMinLaunchNs) more = false;
+        }
+        return LaunchBudget{base, more ? kMinLaunchNs : 0, 0};
+    }
+
     // one loop of the worker; returns false when there is nothing to do
     int loop_once(bool &idle) {
         std::vector<int> admitted, stopped;
         long long spare = 0;
         int short_ctas = 0;                          // CTAs the budget lacked for queued requests
+        bool queued = false;                         // requests still wait after admission
         {
             std::unique_lock<std::mutex> lk(mu);
+            *h_waiting = 0;
             // running requests cancelled since the last chunk: marked stopped
             // on the host and, below, on the device, then retired as finished
             for (uint64_t id : cancels)
@@ -574,6 +596,7 @@ struct ServerImpl {
                 used_ctas += cl;
             }
             idle = running == 0;
+            queued = !queue.empty();
             spare = (long long)cfg.max_slots - used_ctas - (long long)queue.size();
         }
         cudaError_t e;
@@ -599,6 +622,7 @@ struct ServerImpl {
                 return fail("init kernel", e);
         }
         // chunk launch + status read-back
+        *h_budget = launch_budget(queued);
         nvtxRangePushA("lbm_server_chunk");
         if (graph) {
             if ((e = cudaGraphLaunch(graph, stream))) return fail("graph launch", e);
@@ -613,15 +637,6 @@ struct ServerImpl {
         nvtxRangePop();
         if (e) return fail("chunk", e);
         if (h_dbg[0]) return reject_desc();
-        // (a launch with requests still waiting for the next one keeps to its
-        // slowest slot's chunks)
-        {
-            std::unique_lock<std::mutex> lk(mu);
-            *h_budget = queue.empty() && admitted.empty() ? kMinLaunchNs : 0;
-        }
-        for (int s = 0; s < (int)slots.size(); ++s)
-            if (slots[s].busy && h_status[s].state == kSlotRunning)
-                *h_budget = std::max(*h_budget, (unsigned long long)h_status[s].first_ns);
         ++chunks;
         occupancy_sum += used_ctas;
         // retire finished slots
@@ -842,6 +857,7 @@ int lbm_server_create(const lbm_server_cfg *cfg, void *stream, lbm_server **out)
         ck(cudaMallocHost((void **)&S.h_dbg, sizeof(int) * 8));
         ck(cudaMallocAsync((void **)&S.d_budget, sizeof(*S.d_budget), S.stream));
         ck(cudaMallocHost((void **)&S.h_budget, sizeof(*S.h_budget)));
+        ck(cudaMallocHost((void **)&S.h_waiting, sizeof(int)));
         ck(cudaMallocHost((void **)&S.h_desc, sizeof(SlotDesc) * ns));
         ck(cudaMallocHost((void **)&S.h_status, sizeof(SlotStatus) * ns));
         ck(cudaMallocHost((void **)&S.h_idx, sizeof(int) * ns));
@@ -854,7 +870,8 @@ int lbm_server_create(const lbm_server_cfg *cfg, void *stream, lbm_server **out)
             ck(cudaMemcpyAsync(S.d_status, S.h_status, sizeof(SlotStatus) * ns, cudaMemcpyHostToDevice, S.stream));
             ck(cudaMemsetAsync(S.d_dbg, 0, sizeof(int) * 8, S.stream));
             std::memset(S.h_dbg, 0, sizeof(int) * 8);
-            *S.h_budget = kMinLaunchNs;
+            *S.h_budget = LaunchBudget{};
+            *S.h_waiting = 0;
             ck(cudaStreamSynchronize(S.stream));
         }
         if (e == cudaSuccess && cfg->use_graph) {
@@ -902,6 +919,7 @@ int lbm_server_submit(lbm_server *h, const lbm_request *r, uint64_t *id) {
         if (id) *id = p.id;
         S.queue.push_back(p);
         ++S.submitted;
+        *S.h_waiting = 1;
     }
     S.cv_work.notify_one();
     return LBM_OK;
@@ -949,6 +967,7 @@ int lbm_server_cancel(lbm_server *h, uint64_t id) {
         for (const SlotInfo &si : S.slots) running = running || (si.busy && si.id == id);
         if (!running) { set_error("no queued or running request with this id"); return LBM_EINVAL; }
         S.cancels.push_back(id);
+        *S.h_waiting = 1;
     }
     S.cv_work.notify_one();
     return LBM_OK;
@@ -1019,6 +1038,7 @@ int lbm_server_destroy(lbm_server *h) {
     if (!h) return LBM_OK;
     ServerImpl &S = h->s;
     S.stop = true;
+    if (S.h_waiting) *S.h_waiting = 1;
     S.cv_work.notify_all();
     if (S.worker.joinable()) S.worker.join();
     if (S.graph) cudaGraphExecDestroy(S.graph);
@@ -1045,6 +1065,7 @@ int lbm_server_destroy(lbm_server *h) {
     if (S.h_out) cudaFreeHost(S.h_out);
     if (S.h_dbg) cudaFreeHost(S.h_dbg);
     if (S.h_budget) cudaFreeHost(S.h_budget);
+    if (S.h_waiting) cudaFreeHost((void *)S.h_waiting);
     delete h;
     return LBM_OK;
 }
