@@ -2,6 +2,7 @@
 // the host runtime.
 #pragma once
 
+#include "float_pairs.h"
 #include "lbm_internal.h"
 
 namespace lbm {
@@ -71,9 +72,8 @@ struct SlotDesc {
     signed char term_ey[2][32];   // its e_y
     signed char out_a[2][kMaxOut];
     // its re-emission M_in g^w_a / D_w - w_a = c0 + d c with d the sum of the
-    // incoming deviations, c = g^w_a / D_w and c0 = (the terms' weights) c - w_a,
-    // both as pairs of floats
-    KWall::Emit out_e[2][kMaxOut];
+    // incoming deviations, c = g^w_a / D_w and c0 = (the terms' weights) c - w_a
+    Emit3 out_e[2][kMaxOut];
     KConsts<float> k;         // per-instance constants (Nx = 1, pitch = 1)
 };
 

@@ -351,9 +351,9 @@ struct SmemState {
 // 4900 per step, since every FP64 warp instruction takes 64 on GB300.  So the
 // sum of the deviations runs in FP32 with error-free additions (Sum3: to far
 // below FP64's rounding): every group of four lanes sums all terms, seven per
-// lane, then two butterfly stages; and c0 + d c is evaluated in pairs of floats,
-// hi + lo to 2^-46.  terms(t, x) reads the incoming terms t[] of the current state;
-// the wall rows belong to this CTA.
+// lane, then two butterfly stages; and c0 + d c is evaluated in floats to what
+// FP64 keeps of it (emit3).  terms(t, x) reads the incoming terms t[] of the
+// current state; the wall rows belong to this CTA.
 // The FP32 value of each re-emission is rounded stochastically (add_sr of
 // its round-to-nearest value and the FP32 remainder), from the hash of the
 // step and a counter beyond the slot's rows.
@@ -362,7 +362,7 @@ template <class TermFn>
 __device__ __forceinline__ void wall_fill_warp(const SlotDesc &d, int wall, int lane,
                                                float *fill, uint32_t step, TermFn &&terms) {
     const int l = min(lane, d.nout - 1);
-    const KWall::Emit ce = d.out_e[wall][l];
+    const Emit3 ce = d.out_e[wall][l];
     // this lane's terms (lane & 3) + 4 i, all loads in flight; past the last
     // term the loads repeat it
     float x[kLaneTerms];
@@ -377,17 +377,10 @@ __device__ __forceinline__ void wall_fill_warp(const SlotDesc &d, int wall, int 
     for (int o = 1; o <= 2; o <<= 1) {
         const float h = __shfl_xor_sync(0xffffffffu, sum.h, o), m = __shfl_xor_sync(0xffffffffu, sum.m, o),
                     r = __shfl_xor_sync(0xffffffffu, sum.l, o);
-        sum.add(h);
-        sum.add(m);
-        sum.l = __fadd_rn(sum.l, r);
+        sum.add(h, m, r);
     }
-    const float dh = __fadd_rn(sum.h, sum.m);
-    const float dl = __fadd_rn(__fsub_rn(sum.m, __fsub_rn(dh, sum.h)), sum.l);
-    const float p = __fmul_rn(dh, ce.ch), e = __fmaf_rn(dh, ce.ch, -p);
-    float v, r;
-    two_sum(ce.c0h, p, v, r);
-    const float z = __fadd_rn(r, __fadd_rn(ce.c0l, __fmaf_rn(dh, ce.cl, __fmaf_rn(dl, ce.ch, e))));
-    const float hi = __fadd_rn(v, z), lo = __fsub_rn(z, __fsub_rn(hi, v));
+    float hi, lo;
+    emit3(ce, sum, hi, lo);
     const uint32_t h = sr_cell(step, (uint32_t)(d.Ny + wall));
     if (lane < d.nout) fill[d.out_a[wall][l]] = add_sr(hi, lo, sr_bits32(h, lane));
     __syncwarp();

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "float_pairs.h"
 #include "lattice_tables.h"
 #include "lbm_internal.h"
 
@@ -668,8 +669,8 @@ __device__ __forceinline__ typename Store<PREC>::C wall_mix(typename Store<PREC>
 //  * every FP64 warp instruction, conversions and comparisons included, holds
 //    an SM sub-partition's FP64 unit for 64 cycles, and there were about 100
 //    per wall cell (26 terms, 15 re-emissions for D2Q37).  For the FP32 and
-//    BF16 formats the sum runs in FP32 with error-free additions (Knuth's
-//    TwoSum; three floats hold it to far below FP64's rounding) and each
+//    BF16 formats the sum runs in FP32 with error-free additions (Sum3:
+//    three floats hold it to far below FP64's rounding) and each
 //    re-emission is evaluated as c0 + d c in pairs of floats with a bound on its
 //    error; only where the bound straddles an FP32 rounding boundary (about one
 //    in 10^5) is it formed again in FP64.  The result is the FP64 expression rounded to FP32;
@@ -681,20 +682,6 @@ __device__ __forceinline__ typename Store<PREC>::C wall_mix(typename Store<PREC>
 // in FP64; 10.1 in FP32, inlined; 7.8 as a loop; 5.3 with the re-emissions
 // branch-free and the launch overlapped.  4096 x 2048, whose wall blocks end
 // the step: FP32 378 -> 360, BF16SHIFT 262 -> 234; 3001 x 1203 BF16DEV 164 -> 133.
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-struct Sum3 {                                // a running sum h + m + l
-    float h = 0.0f, m = 0.0f, l = 0.0f;
-    __device__ __forceinline__ void add(float x) {
-        float e, e2;
-        two_sum(h, x, h, e);
-        two_sum(m, e, m, e2);
-        l = __fadd_rn(l, e2);
-    }
-};
 
 // The FP64 expressions of a column's re-emissions, from the sum's three floats.
 // Out of line, so that the compiler does not evaluate them along the FP32 ones.

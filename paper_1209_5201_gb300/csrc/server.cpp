@@ -289,7 +289,7 @@ struct ServerImpl {
             const double c = d.k.wcoef[wl][a];
             if (no[wl] >= kMaxOut || !(c > 0.0)) std::abort();
             d.out_a[wl][no[wl]] = (signed char)a;
-            d.out_e[wl][no[wl]++] = wall_emit(c, std::fma(wterm[wl], c, -(double)d.k.w[a]));
+            d.out_e[wl][no[wl]++] = emit3_of(c, wterm[wl], (double)d.k.w[a]);
         }
         if (no[0] != no[1] || no[0] < 1) std::abort();
         d.nout = no[0];
