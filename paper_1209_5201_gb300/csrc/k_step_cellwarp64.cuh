@@ -206,9 +206,10 @@ struct CellLane {
             if (k.eq_order == 3) O = s * __fma_rn(1.0 / 6.0, s2, A1);
         }
         const double orho = om * rho, omc = 1.0 - om;
+        // (the pulled value, the largest term, is added last: one rounding at its size)
         const double P = (orho * we) * E, ow = orho * wo;
-        va = __fma_rn(ow, O, __fma_rn(omc, fa, P));
-        vb = __fma_rn(-ow, O, __fma_rn(omc, fb, P));
+        va = __fma_rn(omc, fa, __fma_rn(ow, O, P));
+        vb = __fma_rn(omc, fb, __fma_rn(-ow, O, P));
         __syncwarp();                        // every lane has read sf
     }
     // the pair into a state buffer, with the halo copies other kernels read
