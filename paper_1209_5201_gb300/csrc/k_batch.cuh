@@ -6,14 +6,14 @@
 //
 // With Nx = 1 the pull of Eq. (5) only shifts in y: f_in(j, a) =
 // f~*(j - e_ay, a).  A slot runs on a cluster of CL CTAs (CL = 1, 2, 4, 8 or
-// 16, fixed by its height): CTA `rank` owns rows [rank R, rank R + R), R =
+// 16): CTA `rank` owns rows [rank R, rank R + R), R =
 // ceil(Ny / CL), and a cluster barrier with release / acquire semantics
-// separates the steps.  When its rows fit (batch_uses_smem) the CTA keeps them in shared
-// memory for the whole launch (loaded from the pool at the start, written back
-// at the end; one ring per velocity, SmemState) and pulls the <= 3 rows it needs
-// from each neighbour through distributed shared memory (ld.shared::cluster);
-// taller blocks keep the state in global memory (L2-resident, two buffers) and
-// read it with ld.global.cg.
+// separates the steps.  When its rows fit (batch_uses_smem) the CTA keeps them in
+// shared memory for the whole launch (loaded from the pool at the start, written
+// back at the end; two buffers up to 256 rows, one ring per velocity up to 512:
+// SmemState) and pulls the <= 3 rows it needs from each neighbour through
+// distributed shared memory (ld.shared::cluster); taller blocks keep the state in
+// global memory (L2-resident, two buffers) and read it with ld.global.cg.
 //
 // Row mapping inside a CTA: warp 0 of the bottom CTA owns the (up to) 32
 // lowest rows and warp 0 (one CTA: warp 1) of the top CTA the 32 highest; each of
@@ -21,11 +21,11 @@
 // FP64 precision in a fixed order - the (velocity, row) terms of the wall's
 // list, built on the host and carried in the slot descriptor - forms the
 // normalised re-emission of every outgoing velocity once, and then updates its
-// rows (branch-free: sources clamped into the
-// slot, the wall's values selected afterwards).  The other rows never need a wall value,
-// so no block barrier separates the wall sums from the bulk update.  Every
-// slot's arithmetic depends only on the slot itself (its cluster size is a
-// function of its height), never on the slot index, the grid or other slots.
+// rows (branch-free: sources clamped into the slot, the wall's values selected
+// afterwards).  The other rows never need a wall value, so no block barrier
+// separates the wall sums from the bulk update (a full ring's first sums excepted:
+// run_steps).  Every slot's arithmetic depends only on the slot itself, never on
+// its cluster size, the slot index, the grid or other slots.
 #pragma once
 
 #include "batch_internal.h"
@@ -350,17 +350,23 @@ struct SmemState {
 // conversions, the product) it took 1200 - 1550 cycles of a lone column's 3300 -
 // 4900 per step, since every FP64 warp instruction takes 64 on GB300.  So the
 // sum of the deviations runs in FP32 with error-free additions (Sum3: to far
-// below FP64's rounding): every group of four lanes sums all terms, seven per
-// lane, then two butterfly stages; and c0 + d c is evaluated in floats to what
+// below FP64's rounding): every group of four lanes sums all terms, up to seven
+// per lane, then two butterfly stages; and c0 + d c is evaluated in floats to what
 // FP64 keeps of it (emit3).  terms(t, x) reads the incoming terms t[] of the
 // current state; the wall rows belong to this CTA.
 // The FP32 value of each re-emission is rounded stochastically (add_sr of
 // its round-to-nearest value and the FP32 remainder), from the hash of the
 // step and a counter beyond the slot's rows.
-constexpr int kLaneTerms = kMaxTerm / 4;
-template <class TermFn>
+template <int Q>
+constexpr int lane_terms() {
+    int n = 0;                               // incoming terms per wall
+    for (int a = 0; a < Q; ++a) n += Lat<Q>::ey(a) > 0 ? Lat<Q>::ey(a) : 0;
+    return (n + 3) / 4;
+}
+template <int Q, class TermFn>
 __device__ __forceinline__ void wall_fill_warp(const SlotDesc &d, int wall, int lane,
                                                float *fill, uint32_t step, TermFn &&terms) {
+    constexpr int kLaneTerms = lane_terms<Q>();
     const int l = min(lane, d.nout - 1);
     const Emit3 ce = d.out_e[wall][l];
     // this lane's terms (lane & 3) + 4 i, all loads in flight; past the last
@@ -435,6 +441,7 @@ __device__ __forceinline__ void run_steps(const SlotDesc &d, State &S, BatchWall
                                           int chunk, int CL, int warp, int lane, int tid,
                                           int nth, int j0, int j1, int nb, int nt, int mb,
                                           int me, uint32_t step0) {
+    constexpr int kLaneTerms = lane_terms<Q>();
     int jw = -1;
     // the top wall's warp: not the bottom wall's, and none of those that the
     // bulk rows of a full CTA with one wall fill
@@ -451,7 +458,7 @@ __device__ __forceinline__ void run_steps(const SlotDesc &d, State &S, BatchWall
     if (wall_warp) {
         for (int t = lane; t < d.nterm; t += 32)
             sw.toff[wall][t] = S.term_off(wall, d.term_a[wall][t], d.term_ey[wall][t], d.term_row[wall][t]);
-        wall_fill_warp(d, wall, lane, sw.fill[wall], step0, [&](const int (&t)[kLaneTerms], float (&x)[kLaneTerms]) {
+        wall_fill_warp<Q>(d, wall, lane, sw.fill[wall], step0, [&](const int (&t)[kLaneTerms], float (&x)[kLaneTerms]) {
 #pragma unroll
             for (int i = 0; i < kLaneTerms; ++i) {
                 const int kk = d.term_row[wall][t[i]];
@@ -468,15 +475,6 @@ __device__ __forceinline__ void run_steps(const SlotDesc &d, State &S, BatchWall
     // read its terms before any warp stores: here for the chunk's first step,
     // before the step's barrier for the others.
     if (!State::kTwoBuffers && CL == 1) __syncthreads();
-    auto fill_next = [&](uint32_t st) {
-        wall_fill_warp(d, wall, lane, sw.fill[wall], st, [&](const int (&t)[kLaneTerms], float (&x)[kLaneTerms]) {
-            int off[kLaneTerms];
-#pragma unroll
-            for (int i = 0; i < kLaneTerms; ++i) off[i] = sw.toff[wall][t[i]];
-#pragma unroll
-            for (int i = 0; i < kLaneTerms; ++i) x[i] = S.term_at(off[i]);
-        });
-    };
     for (int step = 0; step < chunk; ++step) {
         const uint32_t gstep = step0 + (uint32_t)step;
         for (int it = jw >= 0 ? -1 : 0;; ++it) {
@@ -488,31 +486,26 @@ __device__ __forceinline__ void run_steps(const SlotDesc &d, State &S, BatchWall
             const bool edge = __any_sync(__activemask(), j < j0 + 3 || j >= j1 - 3);
             cell_update<Q, PRECISE>(d, S, j, edge, sw, gstep);
         }
-        const bool more = step + 1 < chunk;
-        if (CL == 1) {
-            if constexpr (State::kTwoBuffers) {
-                // while the other warps run ahead: the wall warps' rows then
-                // have their SM sub-partitions to themselves
-                __syncthreads();
-                S.flip();
-                if (wall_warp && more) fill_next(gstep + 1u);
-            } else {
-                // before the barrier: afterwards another warp may store to the
-                // slots (of a ring) of what has left the column
-                __syncwarp();
-                S.flip();
-                if (wall_warp && more) fill_next(gstep + 1u);
-                __syncthreads();
-            }
-        } else {
-            // the next step's wall sums read only rows this warp has just
-            // written (visible to it after __syncwarp), so they run between
-            // arriving at the cluster barrier and waiting on it
-            cluster_arrive();
-            S.flip();
-            if (wall_warp && more) fill_next(gstep + 1u);
-            cluster_wait();
-        }
+        // The next step's wall sums read rows of their own warp alone, visible to
+        // it after __syncwarp, so they run between arriving at the cluster barrier
+        // and waiting on it; on one CTA before the block barrier, for afterwards
+        // another warp may store to the slots (of a ring) of what has left the
+        // column.  One copy of their code serves every case: a lone D2Q25 column
+        // of 256 rows 1.07 us per step, 1.16 with a copy for each.
+        __syncwarp();
+        if (CL > 1) cluster_arrive();
+        S.flip();
+        if (wall_warp && step + 1 < chunk)
+            wall_fill_warp<Q>(d, wall, lane, sw.fill[wall], gstep + 1u,
+                              [&](const int (&t)[kLaneTerms], float (&x)[kLaneTerms]) {
+                int off[kLaneTerms];
+#pragma unroll
+                for (int i = 0; i < kLaneTerms; ++i) off[i] = sw.toff[wall][t[i]];
+#pragma unroll
+                for (int i = 0; i < kLaneTerms; ++i) x[i] = S.term_at(off[i]);
+            });
+        if (CL > 1) cluster_wait();
+        else __syncthreads();
     }
 }
 
