@@ -105,6 +105,8 @@ struct ServerImpl {
     // clusters of kBatchClassCL[c] CTAs, each class launched on its own stream
     int cls_base[kBatchClasses] = {}, cls_cap[kBatchClasses] = {};
     int max_cl = 8;            // largest cluster the device schedules (8 or 16)
+    bool split_any = false;    // clusters for short requests too (the autotuner's
+                               // few steps on each cluster size)
     cudaStream_t side[kBatchClasses] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[kBatchClasses] = {};
     int *d_idx = nullptr;                    // slot lists for init / read-out
@@ -363,7 +365,7 @@ struct ServerImpl {
         cl = batch_cluster_size(r.Ny, cfg.cluster_rows, cfg.max_slots, max_cl);
         if (cl == 1) return false;
         work = std::min(est_steps(r), (double)r.max_steps) * std::ceil(r.Ny / 256.0);
-        return work >= least;
+        return split_any || work >= least;
     }
 
     // the cluster whose CTAs hold a column's rows in shared memory (1 where a
@@ -797,7 +799,7 @@ int lbm_request_bytes(const lbm_request *r, size_t *bytes) {
     return LBM_OK;
 }
 
-int lbm_server_create(const lbm_server_cfg *cfg, void *stream, lbm_server **out) {
+static int server_create(const lbm_server_cfg *cfg, void *stream, bool split_any, lbm_server **out) {
     try {
         if (!cfg || !out) { set_error("NULL argument"); return LBM_EINVAL; }
         *out = nullptr;
@@ -814,6 +816,7 @@ int lbm_server_create(const lbm_server_cfg *cfg, void *stream, lbm_server **out)
         lbm_server *h = new lbm_server;
         ServerImpl &S = h->s;
         S.cfg = *cfg;
+        S.split_any = split_any;
         S.stream = (cudaStream_t)stream;
         S.t0 = std::chrono::steady_clock::now();
         cudaGetDevice(&S.device);
@@ -902,6 +905,10 @@ int lbm_server_create(const lbm_server_cfg *cfg, void *stream, lbm_server **out)
         set_error("server creation failed");
         return LBM_ENOMEM;
     }
+}
+
+int lbm_server_create(const lbm_server_cfg *cfg, void *stream, lbm_server **out) {
+    return server_create(cfg, stream, false, out);
 }
 
 int lbm_server_submit(lbm_server *h, const lbm_request *r, uint64_t *id) {
@@ -1096,12 +1103,13 @@ int lbm_batch_solve(const lbm_server_cfg *cfg, void *stream, const lbm_request *
 namespace {
 
 // Wall seconds from the first submit to the drain of n identical fixed-step
-// requests (lattice kind, Ny rows, Kn, walls -+0.1, tol 0: never converged)
-// on a server with cfg; *cell_steps gets the lattice updates they ran.
+// requests (lattice kind, Ny rows, Kn, walls -+0.1, tol 0: never converged) on a
+// server with cfg that splits any request; *cell_steps gets the lattice updates
+// they ran.
 int time_fixed_steps(const lbm_server_cfg &cfg, void *stream, int kind, int Ny, double Kn, int n,
                      int64_t steps, double *seconds, double *cell_steps) {
     lbm_server *h = nullptr;
-    if (int rc = lbm_server_create(&cfg, stream, &h)) return rc;
+    if (int rc = server_create(&cfg, stream, true, &h)) return rc;
     lbm_request r;
     std::memset(&r, 0, sizeof(r));
     r.lattice = kind;
@@ -1153,9 +1161,9 @@ extern "C" int lbm_server_autotune(lbm_server_cfg *cfg, void *stream, lbm_server
     }
     const int max_cl = batch_max_cluster();
     // ---- lone columns on every usable cluster size --------------------------
-    // a lone long request (small Kn) gets the largest usable cluster within the
-    // CTA budget: the budget picks the cluster size; long chunks keep the
-    // host's per-launch work out of the step time
+    // a lone request of these servers gets the largest usable cluster within the
+    // CTA budget, however few its steps: the budget picks the cluster size; long
+    // chunks keep the host's per-launch work out of the step time
     auto lone_us = [&](int kind, int Ny, int cl, double *us) -> int {
         *us = 0.0;
         if (cl > max_cl || batch_cluster_size(Ny, 32, cl, max_cl) != cl) return LBM_OK;
