@@ -11,7 +11,7 @@
 //
 // Bound by its FP64 instructions (64 cycles each per warp and SM sub-partition
 // on GB300).  Forming f_a, its division and the central products velocity by
-// velocity took about 1900 of them per cell; here about 320: the sums over the
+// velocity took about 1900 of them per cell; here 369 (counted, conversions too): the sums over the
 // velocities are raw moments of f~ (sums and differences of opposite pairs,
 // integer factors), f^eq enters through its moments alone - it is w_a times a
 // polynomial in the integer velocity, so they are its 15 coefficients times

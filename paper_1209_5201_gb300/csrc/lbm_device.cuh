@@ -679,7 +679,7 @@ __device__ __forceinline__ typename Store<PREC>::C wall_mix(typename Store<PREC>
 //    had no time to cache.  One copy serves both walls (velocity and opposite),
 //    the re-emissions are a loop, the pull reads its fill from shared memory.
 // D2Q37 FP32 on 300 x 40 (a step as long as its wall blocks), us per step: 19.1
-// in FP64; 10.1 in FP32, inlined; 7.8 as a loop; 5.3 with the re-emissions
+// in FP64; 10.1 in FP32, inlined; 7.8 as a loop; 5.3 - 5.7 with the re-emissions
 // branch-free and the launch overlapped.  4096 x 2048, whose wall blocks end
 // the step: FP32 378 -> 360, BF16SHIFT 262 -> 234; 3001 x 1203 BF16DEV 164 -> 133.
 
