@@ -36,10 +36,14 @@ def test_short_request_beside_a_long_one(lbm, use_graph):
             if rid in done:
                 break
         ms.append(1e3 * (time.perf_counter() - t))
-    t = time.perf_counter()
-    s.cancel(bg)
-    while not s.poll(8):
-        pass
-    cancel = 1e3 * (time.perf_counter() - t)
+    cancels = []
+    for _ in range(5):
+        t = time.perf_counter()
+        s.cancel(bg)
+        while not s.poll(8):
+            pass
+        cancels.append(1e3 * (time.perf_counter() - t))
+        bg = s.submit(lbm.make_request("D2Q37", 256, 0.002, 0.1, tol=1e-30, max_steps=10_000_000))
+        time.sleep(0.02 + rng.uniform(0.0, 0.004))
     s.close()
-    assert np.median(ms) < 1.0 and cancel < 1.5, (ms, cancel)
+    assert np.median(ms) < 1.0 and np.median(cancels) < 1.0, (ms, cancels)
