@@ -529,9 +529,10 @@ typedef struct lbm_server_tuning {
  * chunks a cluster slot runs while a one-CTA slot runs one, 1..16);
  * cluster_rows = the median over lattices and heights of the rows per CTA
  * of the smallest cluster within 15 % of the fastest (32 .. 1024); and
- * chunk_steps = the longest chunk within 5 % of the best full-GPU rate
- * (fewer launches, each a host round trip).  Takes about half a minute;
- * the device must be otherwise idle for the times to mean anything.  `stream`
+ * chunk_steps = of the chunks that end within 2 ms on a full GPU the longest
+ * within 5 % of their best rate (a launch runs several shorter ones; arrivals
+ * and step limits wait for the end of a longer one).  Takes about half a minute; the
+ * device must be otherwise idle for the times to mean anything.  `stream`
  * as for lbm_server_create; `report` (may be NULL) receives the times.
  * Results of a solve do not depend on cluster_rows or class_sub; chunk_steps
  * moves the steps at which its convergence checks fall.

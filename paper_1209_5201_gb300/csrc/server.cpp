@@ -88,6 +88,17 @@ int lattice_q(int kind) {
     return kind == LBM_LATTICE_D2Q17 ? 17 : kind == LBM_LATTICE_D2Q37 ? 37 : 25;
 }
 
+// Steps per chunk of a column: cheaper slots run more steps, so that every CTA
+// of a launch takes about as long (chunk_steps x 333 cost units); the cost model
+// is the velocity count times the rows per thread of one 256-thread CTA plus a
+// latency floor.  It ignores the cluster on purpose: chunk lengths and residual
+// checks then fall on the same steps however the column is split.
+int chunk_length(int Q, int Ny, int chunk_steps) {
+    const double cost = Q * std::ceil(Ny / 256.0) + 37.0, cost_ref = 37.0 * 8.0 + 37.0;
+    return (int)std::min<double>(32.0 * chunk_steps,
+                                 std::max<double>(chunk_steps, std::round(chunk_steps * cost_ref / cost)));
+}
+
 }  // namespace
 
 struct ServerImpl {
@@ -221,17 +232,7 @@ struct ServerImpl {
         d.cur = 0;
         d.cl = cl;
         d.sub = sub_for(cl);
-        // Steps per chunk launch: cheaper slots run more steps, so that every
-        // CTA of a launch takes about as long (cfg.chunk_steps x 333 cost
-        // units); the cost model is the velocity count times the rows per
-        // thread of one 256-thread CTA plus a latency floor.  It ignores the
-        // cluster on purpose: chunk lengths and residual checks then fall on
-        // the same steps however the column is split.
-        const double cost = L.Q * std::ceil(r.Ny / 256.0) + 37.0;
-        const double cost_ref = 37.0 * 8.0 + 37.0;
-        d.chunk_steps = (int)std::min<double>(32.0 * cfg.chunk_steps,
-                                              std::max<double>(cfg.chunk_steps,
-                                                               std::round(cfg.chunk_steps * cost_ref / cost)));
+        d.chunk_steps = chunk_length(L.Q, r.Ny, cfg.chunk_steps);
         // residual every ~quarter of the slowest e-folding time of the start-up
         // (0.127 Ny r / Kn steps for the fundamental shear mode), in chunks
         const double efold = r.tau > 0 ? r.Ny * r.Ny / (9.8696 * r.tau * L.r * r.Ny)
@@ -1214,7 +1215,11 @@ extern "C" int lbm_server_autotune(lbm_server_cfg *cfg, void *stream, lbm_server
     // ---- chunk length on a full GPU of one-CTA columns ------------------------
     // (D2Q37, 256 rows: the heaviest one-CTA column; best of two runs each)
     const int chunks[5] = {25, 50, 100, 200, 400};
-    double best = 0;
+    double best = 0;                         // of the chunks that end within a launch
+    auto in_time = [&](int i) {
+        return chunk_length(37, 256, chunks[i]) * 256.0 * cfg->max_slots <=
+               (double)kMinLaunchNs * rep.chunk_glups[i];
+    };
     for (int i = 0; i < 5; ++i) {
         lbm_server_cfg lc = *cfg;
         lc.cluster_rows = kMaxNy;
@@ -1228,13 +1233,19 @@ extern "C" int lbm_server_autotune(lbm_server_cfg *cfg, void *stream, lbm_server
                 return rc;
             rep.chunk_glups[i] = std::max(rep.chunk_glups[i], sec > 0 ? cells / sec / 1e9 : 0.0);
         }
-        best = std::max(best, rep.chunk_glups[i]);
+        if (in_time(i)) best = std::max(best, rep.chunk_glups[i]);
     }
-    // the longest chunk within 5 % of the best rate: fewer launches (each
-    // costs the host a round trip) at about the same rate
+    // of the chunks that end within a launch (kMinLaunchNs, which shorter ones fill
+    // by several) the longest within 5 % of their best rate: each chunk has a
+    // residual check's and a decision's overhead, but a longer one is only what
+    // arrivals and step limits wait for.  304 CTAs, chunk lengths 25 / 50 / 100 / 200 /
+    // 400: a lone 4096-row D2Q37 column 1.80 / 1.77 / 1.75 / 1.73 / 1.71 us per step, a
+    // 450-step request beside one of 2048 rows 1.5 / 1.5 / 1.5 / 3.4 / 5.8 ms, 304 mixed
+    // solves at once 0.40 / 0.36 / 0.35 / 0.37 / 0.41 s.  (The shortest where none ends
+    // in time.)
     int chunk = chunks[0];
     for (int i = 0; i < 5; ++i)
-        if (rep.chunk_glups[i] >= 0.95 * best) chunk = chunks[i];
+        if (in_time(i) && rep.chunk_glups[i] >= 0.95 * best) chunk = chunks[i];
     // ---- the choices ------------------------------------------------------------
     cfg->chunk_steps = chunk;
     cfg->class_sub[0] = 1;
